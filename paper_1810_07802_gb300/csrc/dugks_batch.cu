@@ -55,6 +55,21 @@ struct Group {
     int nwork = 0;
 };
 
+// Members stepped by the strip kernel, grouped by precision, model and y-boundary.  A group's launch carries the
+// constants of at most kStripMembers members, so a larger group is several launches a step.
+struct StripMembers {
+    bool fp32 = false, coupled = false, wally = false;
+    std::vector<dugks_ctx *> members;
+    std::vector<int2> size;              // strips across, rows
+    std::vector<dugks::Phys<float>> ph32;
+    std::vector<dugks::StripPhys<double>> ph64;
+    std::vector<unsigned char> h_inst;
+    void *d_inst = nullptr;
+    size_t cap = 0;
+    int rows = 1;                        // rows of a chunk
+    int parts() const { return ((int)members.size() + dugks::kStripMembers - 1) / dugks::kStripMembers; }
+};
+
 size_t desc_size(bool fp32) { return fp32 ? sizeof(InstDesc<float>) : sizeof(InstDesc<double>); }
 
 dugks_status from_cuda(cudaError_t e) {
@@ -70,6 +85,10 @@ struct dugks_batch_ctx {
     std::vector<dugks_ctx *> solo;   // members stepped by the single-problem kernel
     bool grouped = false;            // some group is non-empty
     static constexpr int kGroups = 16 * kMaxTiles;
+    StripMembers strips[8];          // index: fp32 * 4 + coupled * 2 + wally
+    // groups step independently of one another: each is a branch of the captured graph
+    std::vector<cudaStream_t> side;
+    std::vector<cudaEvent_t> done;   // [0]: the fork, [1 + i]: branch i
     Group groups[kGroups];   // index: (upw * 8 + fp32 * 4 + coupled * 2 + wally) * kMaxTiles + tile
     bool dirty = true;
     bool persistent = false;         // K steps per launch (else one grid launch per step)
@@ -83,6 +102,69 @@ struct dugks_batch_ctx {
         exec = exec_k = nullptr;
     }
 
+    // The strip members of one kind: their sizes and constants when dirty, their descriptors always.
+    template <typename Real>
+    cudaError_t upload_strips(int i, std::vector<typename dugks::StripConst<Real>::T> &ph) {
+        StripMembers &g = strips[i];
+        if (dirty) {
+            g.fp32 = i & 4;
+            g.coupled = i & 2;
+            g.wally = i & 1;
+            g.members.clear();
+            g.size.clear();
+            ph.clear();
+            for (dugks_ctx *c : members)
+                if (c->strip.threads && c->fp32 == g.fp32 && c->coupled == g.coupled && c->wally == g.wally &&
+                    member_tiles(c) < kSoloTiles) {
+                    g.members.push_back(c);
+                    g.size.push_back(make_int2(c->strip.nstrips, c->P.ny));
+                    if constexpr (sizeof(Real) == 4) ph.push_back(c->phf);
+                    else ph.push_back(c->spd);
+                }
+            grouped = grouped || !g.members.empty();
+            if (!g.members.empty()) {
+                cudaError_t e = dugks::strip_group_rows<Real>(g.coupled, g.wally, g.size.data(), (int)g.size.size(), &g.rows);
+                if (e != cudaSuccess) return e;
+            }
+        }
+        if (g.members.empty()) return cudaSuccess;
+        using Inst = dugks::StripInst<Real>;
+        g.h_inst.resize(sizeof(Inst) * g.members.size());
+        for (size_t m = 0; m < g.members.size(); m++) {
+            const dugks_ctx *c = g.members[m];
+            if constexpr (sizeof(Real) == 4) dugks::fill_strip_inst(reinterpret_cast<Inst *>(g.h_inst.data()) + m, c, c->phf);
+            else dugks::fill_strip_inst(reinterpret_cast<Inst *>(g.h_inst.data()) + m, c, c->phd);
+        }
+        if (g.h_inst.size() > g.cap) {
+            drop_graph();
+            if (g.d_inst) cudaFree(g.d_inst);
+            g.cap = std::max(g.h_inst.size(), 2 * g.cap);
+            cudaError_t e = cudaMalloc(&g.d_inst, g.cap);
+            if (e != cudaSuccess) {
+                g.d_inst = nullptr;
+                g.cap = 0;
+                return e;
+            }
+        }
+        return cudaMemcpyAsync(g.d_inst, g.h_inst.data(), g.h_inst.size(), cudaMemcpyHostToDevice, st);
+    }
+
+    // k steps of members [first, first + n) of a strip group: one launch a step, each overlapping the end of the
+    // one before, then the advance of their descriptors.
+    template <typename Real>
+    cudaError_t enqueue_strips(const StripMembers &g, const std::vector<typename dugks::StripConst<Real>::T> &ph, int part, int k,
+                               cudaStream_t to) {
+        const int first = part * dugks::kStripMembers;
+        const int n = std::min((int)g.members.size() - first, dugks::kStripMembers);
+        auto *inst = static_cast<dugks::StripInst<Real> *>(g.d_inst) + first;
+        for (int j = 0; j < k; j++) {
+            cudaError_t e = dugks::launch_strip_group<Real>(inst, ph.data() + first, g.size.data() + first, n, g.rows, j,
+                                                            g.coupled, g.wally, j > 0, to);
+            if (e != cudaSuccess) return e;
+        }
+        return dugks::launch_strip_advance<Real>(inst, n, k, to);
+    }
+
     // Rebuilds the host images (descriptors always, work lists when dirty) and uploads them.
     cudaError_t upload() {
         if (dirty) {
@@ -90,6 +172,10 @@ struct dugks_batch_ctx {
             for (dugks_ctx *c : members)
                 if (member_tiles(c) >= kSoloTiles) solo.push_back(c);
             grouped = false;
+        }
+        for (int i = 0; i < 8; i++) {
+            cudaError_t e = (i & 4) ? upload_strips<float>(i, strips[i].ph32) : upload_strips<double>(i, strips[i].ph64);
+            if (e != cudaSuccess) return e;
         }
         for (int gi = 0; gi < kGroups; gi++) {
             Group &g = groups[gi];
@@ -103,7 +189,7 @@ struct dugks_batch_ctx {
                 g.members.clear();
                 for (dugks_ctx *c : members)
                     if (c->fp32 == g.fp32 && c->coupled == g.coupled && c->wally == g.wally && c->tile == g.tile &&
-                        c->upw == g.upw && member_tiles(c) < kSoloTiles)
+                        c->upw == g.upw && !c->strip.threads && member_tiles(c) < kSoloTiles)
                         g.members.push_back(c);
                 grouped = grouped || !g.members.empty();
                 const int tx = g.fp32 ? dugks::tile_dim<float>(g.tile, 0) : dugks::tile_dim<double>(g.tile, 0);
@@ -160,20 +246,49 @@ struct dugks_batch_ctx {
         return cudaSuccess;
     }
 
-    // k batched steps: every non-empty group's launches and descriptor advances.
+    int branches() const {
+        int n = 0;
+        for (const Group &g : groups) n += !g.members.empty();
+        for (const StripMembers &g : strips) n += g.parts();
+        return n;
+    }
+
+    // k batched steps: every non-empty group's launches and descriptor advances, each group a branch of its own.
     cudaError_t enqueue_steps(int k) {
+        const int nb = branches();
+        int b = 0;
+        cudaError_t e = cudaSuccess;
+        if (nb > 1) e = cudaEventRecord(done[0], st);
+        auto branch = [&](auto &&launches) {
+            if (e != cudaSuccess) return;
+            if (nb == 1) {
+                e = launches(st);
+                return;
+            }
+            e = cudaStreamWaitEvent(side[b], done[0], 0);
+            if (e == cudaSuccess) e = launches(side[b]);
+            if (e == cudaSuccess) e = cudaEventRecord(done[1 + b], side[b]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, done[1 + b], 0);
+            b++;
+        };
+        for (StripMembers &g : strips)
+            for (int p = 0; p < g.parts(); p++)
+                branch([&](cudaStream_t to) {
+                    return g.fp32 ? enqueue_strips<float>(g, g.ph32, p, k, to) : enqueue_strips<double>(g, g.ph64, p, k, to);
+                });
         for (Group &g : groups) {
             if (g.members.empty()) continue;
             unsigned *ctr = persistent ? g.d_ctr : nullptr;
-            cudaError_t e = g.fp32 ? dugks::launch_batch_step<float>(g.tile, g.upw, static_cast<InstDesc<float> *>(g.d_desc),
-                                                                     g.d_work, g.nwork, (int)g.members.size(),
-                                                                     g.coupled, g.wally, k, ctr, st)
-                                   : dugks::launch_batch_step<double>(g.tile, g.upw, static_cast<InstDesc<double> *>(g.d_desc),
-                                                                      g.d_work, g.nwork, (int)g.members.size(),
-                                                                      g.coupled, g.wally, k, ctr, st);
-            if (e != cudaSuccess) return e;
+            branch([&](cudaStream_t to) {
+                return g.fp32 ? dugks::launch_batch_step<float>(g.tile, g.upw, static_cast<InstDesc<float> *>(g.d_desc),
+                                                                g.d_work, g.nwork, (int)g.members.size(), g.coupled,
+                                                                g.wally, k, ctr, to)
+                              : dugks::launch_batch_step<double>(g.tile, g.upw, static_cast<InstDesc<double> *>(g.d_desc),
+                                                                 g.d_work, g.nwork, (int)g.members.size(), g.coupled,
+                                                                 g.wally, k, ctr, to);
+            });
         }
-        return cudaSuccess;
+        return e;
     }
 
     // Captures `steps` consecutive batched steps into one executable graph.
@@ -183,6 +298,19 @@ struct dugks_batch_ctx {
             cudaError_t e = g.fp32 ? dugks::batch_prepare<float>(g.tile, g.coupled, g.wally, g.upw)
                                    : dugks::batch_prepare<double>(g.tile, g.coupled, g.wally, g.upw);
             if (e != cudaSuccess) return e;
+        }
+        const size_t nb = (size_t)branches();
+        while (nb > 1 && side.size() < nb) {
+            cudaStream_t t = nullptr;
+            cudaError_t e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
+            if (e != cudaSuccess) return e;
+            side.push_back(t);
+        }
+        while (nb > 1 && done.size() < nb + 1) {
+            cudaEvent_t t = nullptr;
+            cudaError_t e = cudaEventCreateWithFlags(&t, cudaEventDisableTiming);
+            if (e != cudaSuccess) return e;
+            done.push_back(t);
         }
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
@@ -242,11 +370,14 @@ dugks_status dugks_batch_step(dugks_batch b, int64_t nsteps) {
         for (int64_t n = 0; n < rest && e == cudaSuccess; n++) e = cudaGraphLaunch(b->exec, b->st);
     }
     if (e != cudaSuccess) return from_cuda(e);
+    auto advance = [&](dugks_ctx *c) {
+        c->steps += nsteps;
+        c->cur ^= (int)(nsteps & 1);
+    };
     for (Group &g : b->groups)
-        for (dugks_ctx *c : g.members) {
-            c->steps += nsteps;
-            c->cur ^= (int)(nsteps & 1);
-        }
+        for (dugks_ctx *c : g.members) advance(c);
+    for (StripMembers &g : b->strips)
+        for (dugks_ctx *c : g.members) advance(c);
     // large members: their own launches, on the batch's stream, in member order
     for (dugks_ctx *c : b->solo) {
         e = dugks::step_on(c, nsteps, b->st);
@@ -288,6 +419,10 @@ dugks_status dugks_batch_destroy(dugks_batch b) {
         if (g.d_work) cudaFree(g.d_work);
         if (g.d_ctr) cudaFree(g.d_ctr);
     }
+    for (StripMembers &g : b->strips)
+        if (g.d_inst) cudaFree(g.d_inst);
+    for (cudaStream_t t : b->side) cudaStreamDestroy(t);
+    for (cudaEvent_t t : b->done) cudaEventDestroy(t);
     delete b;
     return from_cuda(e);
 }

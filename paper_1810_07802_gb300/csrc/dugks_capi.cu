@@ -86,7 +86,14 @@ cudaError_t launch_reduce(const double *phi, const double *ux, const double *uy,
 cudaError_t step_on(dugks_ctx *c, long long nsteps, cudaStream_t st) {
     for (long long n = 0; n < nsteps; n++) {
         cudaError_t e;
-        if (c->fp32)
+        if (c->strip.threads) {
+            if (c->fp32)
+                e = launch_strip<float>(c->strip, c->strip_maps[c->cur], c->step_args<float>(), c->phf, c->phf, c->coupled,
+                                        c->wally, st);
+            else
+                e = launch_strip<double>(c->strip, c->strip_maps[c->cur], c->step_args<double>(), c->spd, c->phd,
+                                         c->coupled, c->wally, st);
+        } else if (c->fp32)
             e = launch_step<float>(c->tile, c->upw, c->tm_state[c->cur], c->tm_hist[c->cur], c->step_args<float>(),
                                    c->phf, c->coupled, c->wally, st);
         else
@@ -374,6 +381,28 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
             c->tma_ok = c->tma_ok && make_box_map(&c->tm_hist[b], c->hist(b), !c->fp32, params->nx, params->ny,
                                                   L.pitch, 2, tx + 8, box_rows);
         }
+    }
+    if (params->tile_shape == 0 && !c->upw) {
+        const cudaError_t es = c->fp32 ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
+                                       : dugks::strip_plan<double>(c->coupled, c->wally, params->nx, params->ny, &c->strip);
+        if (es != cudaSuccess) {
+            if (c->owns) cudaFree(c->ws);
+            delete c;
+            return from_cuda(es);
+        }
+        c->spd = dugks::strip_phys<double>(c->phd);
+        bool ok = true;
+        for (int b = 0; b < 2; b++) {
+            dugks::StripMaps &m = c->strip_maps[b];
+            auto map = [&](CUtensorMap *t, void *base, int planes, int box) {
+                ok = ok && make_box_map(t, base, !c->fp32, params->nx, params->ny, L.pitch, planes, box, 1);
+            };
+            map(&m.src_state, c->state(b), L.nq, c->strip.box);
+            map(&m.src_hist, c->hist(b), 2, c->strip.box);
+            map(&m.dst_state, c->state(b ^ 1), L.nq, c->strip.own);
+            map(&m.dst_hist, c->hist(b ^ 1), 2, c->strip.own);
+        }
+        if (!ok) c->strip.threads = 0;   // no tensor maps: the tile kernels step this problem with plain loads
     }
     cudaError_t e = cudaMemsetAsync(c->ws, 0, L.off_stage, c->st);  // state, history (incl. row padding)
     const size_t fb = L.n * sizeof(double);

@@ -167,11 +167,24 @@ struct Pt {
     Real Dx, Dy;
 };
 
-__device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
+// FP32 takes the hardware's approximations as they are: their arguments (|grad phi|^2 + 1e-16, densities,
+// viscosities, relaxation times) stay clear of the denormals and of 2^126, where alone rsqrtf and __fdividef
+// (1, x) rescale around the same instructions.  FP64: rsqrt and IEEE division.
+__device__ __forceinline__ float rsqrt_r(float x) {
+    float y = x;
+#ifdef __CUDA_ARCH__
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+#endif
+    return y;
+}
 __device__ __forceinline__ double rsqrt_r(double x) { return rsqrt(x); }
-// Reciprocal: the FP32 path uses the fast hardware reciprocal (a few ulp),
-// the FP64 path IEEE division.
-__device__ __forceinline__ float rcp_r(float x) { return __fdividef(1.0f, x); }
+__device__ __forceinline__ float rcp_r(float x) {
+    float y = x;
+#ifdef __CUDA_ARCH__
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+#endif
+    return y;
+}
 __device__ __forceinline__ double rcp_r(double x) { return 1.0 / x; }
 __device__ __forceinline__ float sinpi_r(float x) { return sinpif(x); }
 __device__ __forceinline__ double sinpi_r(double x) { return sinpi(x); }

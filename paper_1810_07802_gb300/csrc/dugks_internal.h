@@ -11,6 +11,7 @@
 
 #include "dugks.h"
 #include "dugks_device.cuh"
+#include "dugks_strip.cuh"
 
 namespace dugks {
 
@@ -20,6 +21,27 @@ template <typename Real> struct InstDesc;
 template <typename Real>
 cudaError_t launch_step(int tile, bool upw, const CUtensorMap &tm_state, const CUtensorMap &tm_hist,
                         const StepArgs<Real> &a, const Phys<Real> &ph, bool coupled, bool wally, cudaStream_t st);
+// Launch geometry of the strip kernel for one problem.
+struct StripPlan {
+    int threads = 0;   // columns of a strip with its halo, one thread each (0: the tile kernels step this problem)
+    int box = 0;       // columns of a staged row
+    int own = 0;       // columns of a finished row
+    int rows = 0;      // rows of a chunk
+    int nstrips = 0;
+    int ctas = 0;      // CTAs that run at once
+};
+template <typename Real>
+cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out);
+template <typename Real>
+cudaError_t launch_strip(const StripPlan &pl, const StripMaps &tm, const StepArgs<Real> &a, const typename StripConst<Real>::T &sp,
+                         const Phys<Real> &ph, bool coupled, bool wally, cudaStream_t st);
+template <typename Real>
+cudaError_t strip_group_rows(bool coupled, bool wally, const int2 *members, int n, int *rows);
+template <typename Real>
+cudaError_t launch_strip_group(const StripInst<Real> *inst, const typename StripConst<Real>::T *ph, const int2 *members, int n,
+                               int rows, int step, bool coupled, bool wally, bool overlap, cudaStream_t st);
+template <typename Real>
+cudaError_t launch_strip_advance(StripInst<Real> *inst, int n, int k, cudaStream_t st);
 template <typename Real>
 int step_box_rows(int tile, bool upw);
 template <typename Real>
@@ -74,6 +96,9 @@ struct dugks_ctx {
     dugks::Phys<float> phf;
     bool tma_ok;
     CUtensorMap tm_state[2], tm_hist[2];
+    dugks::StripPlan strip;
+    dugks::StripMaps strip_maps[2];   // of a step from buffer 0 or 1
+    dugks::StripPhys<double> spd;
 
     void *state(int b) const { return ws + L.off_state[b]; }
     void *hist(int b) const { return ws + L.off_hist[b]; }
@@ -152,5 +177,26 @@ inline void fill_desc(InstDesc<Real> *d, const dugks_ctx *c, const Phys<Real> &p
     d->use_tma = c->tma_ok ? 1 : 0;
     d->vel = static_cast<const Real *>(c->vel());
     d->vel_faces = c->vel_faces;
+}
+
+template <typename Real>
+inline void fill_strip_inst(StripInst<Real> *d, const dugks_ctx *c, const Phys<Real> &ph) {
+    std::memset(static_cast<void *>(d), 0, sizeof *d);
+    for (int b = 0; b < 2; b++) {
+        d->maps[b] = c->strip_maps[b];
+        d->state[b] = static_cast<Real *>(c->state(b));
+        d->hist[b] = static_cast<Real *>(c->hist(b));
+    }
+    d->vel = static_cast<const Real *>(c->vel());
+    d->status = c->status();
+    d->pv = ph;
+    d->plane = (long long)c->L.plane;
+    d->steps = c->steps;
+    d->nx = c->P.nx;
+    d->ny = c->P.ny;
+    d->pitch = c->L.pitch;
+    d->nstrips = c->strip.nstrips;
+    d->vel_faces = c->vel_faces;
+    d->cur = c->cur;
 }
 }  // namespace dugks
