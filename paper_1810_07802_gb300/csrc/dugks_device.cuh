@@ -186,6 +186,9 @@ __device__ __forceinline__ float rcp_r(float x) {
     return y;
 }
 __device__ __forceinline__ double rcp_r(double x) { return 1.0 / x; }
+// a b - c; FP32 in one rounding in every kernel (left to the compiler, tile cells and their halo ring differed).
+__device__ __forceinline__ float mul_sub(float a, float b, float c) { return __fmaf_rn(a, b, -c); }
+__device__ __forceinline__ double mul_sub(double a, double b, double c) { return a * b - c; }
 __device__ __forceinline__ float sinpi_r(float x) { return sinpif(x); }
 __device__ __forceinline__ double sinpi_r(double x) { return sinpi(x); }
 __device__ __forceinline__ float cospi_r(float x) { return cospif(x); }
@@ -1063,8 +1066,8 @@ __device__ __forceinline__ void cell_item(const StepArgs<Real> &a, const Phys<Re
         s.Dx = Real(0);
         s.Dy = Real(0);
     } else {
-        s.Dx = (phux - box[S::off_hbox + e]) * ph.inv_dt;
-        s.Dy = (phuy - box[S::off_hbox + BXY + e]) * ph.inv_dt;
+        s.Dx = mul_sub(s.phi, s.ux, box[S::off_hbox + e]) * ph.inv_dt;
+        s.Dy = mul_sub(s.phi, s.uy, box[S::off_hbox + BXY + e]) * ph.inv_dt;
     }
     st4(aux + c1 * AS, s.dpx, s.dpy, s.lap, s.Dx);
     if (S::F64) aux[c1 * AS + 4] = s.Dy; else sdy[c1] = s.Dy;

@@ -1389,9 +1389,8 @@ __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArg
                 s.Dx = 0.0f;
                 s.Dy = 0.0f;
             } else {
-                // (phi u in one rounding: the tile kernels round it first for their own cells)
-                s.Dx = __fmaf_rn(s.phi, s.ux, -c[HO]) * ph.inv_dt;
-                s.Dy = __fmaf_rn(s.phi, s.uy, -c[HO + BW]) * ph.inv_dt;
+                s.Dx = mul_sub(s.phi, s.ux, c[HO]) * ph.inv_dt;
+                s.Dy = mul_sub(s.phi, s.uy, c[HO + BW]) * ph.inv_dt;
             }
             npu = f2(phux, phuy);
             nr.dp = f2(s.dpx, s.dpy);
