@@ -86,7 +86,9 @@ cudaError_t launch_reduce(const double *phi, const double *ux, const double *uy,
 cudaError_t step_on(dugks_ctx *c, long long nsteps, cudaStream_t st) {
     for (long long n = 0; n < nsteps; n++) {
         cudaError_t e;
-        if (c->strip.threads) {
+        if (c->patch.tx) {
+            e = launch_patch(c->patch, c->step_args<double>(), c->spd, c->phd, c->coupled, c->wally, st);
+        } else if (c->strip.threads) {
             if (c->fp32)
                 e = launch_strip<float>(c->strip, c->strip_maps[c->cur], c->step_args<float>(), c->phf, c->phf, c->coupled,
                                         c->wally, st);
@@ -383,8 +385,10 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
         }
     }
     if (params->tile_shape == 0 && !c->upw) {
-        const cudaError_t es = c->fp32 ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
+        cudaError_t es = c->fp32 ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
                                        : dugks::strip_plan<double>(c->coupled, c->wally, params->nx, params->ny, &c->strip);
+        if (es == cudaSuccess && !c->fp32)
+            es = dugks::patch_plan(c->coupled, c->wally, params->nx, params->ny, c->strip.rows, &c->patch);
         if (es != cudaSuccess) {
             if (c->owns) cudaFree(c->ws);
             delete c;

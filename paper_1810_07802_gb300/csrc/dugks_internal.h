@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <cstring>
+#include <mutex>
 
 #include "dugks.h"
 #include "dugks_device.cuh"
@@ -21,6 +22,22 @@ template <typename Real> struct InstDesc;
 template <typename Real>
 cudaError_t launch_step(int tile, bool upw, const CUtensorMap &tm_state, const CUtensorMap &tm_hist,
                         const StepArgs<Real> &a, const Phys<Real> &ph, bool coupled, bool wally, cudaStream_t st);
+// A value set up once per device (kernel attributes belong to the device's context), by whichever thread comes first.
+template <typename T>
+struct OncePerDevice {
+    static constexpr int kDevices = 64;
+    std::once_flag once[kDevices];
+    T value[kDevices] = {};
+    cudaError_t result[kDevices] = {};
+    template <typename F>
+    cudaError_t get(int dev, T *out, F &&f) {
+        if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
+        std::call_once(once[dev], [&] { result[dev] = f(&value[dev]); });
+        if (out) *out = value[dev];
+        return result[dev];
+    }
+};
+
 // Launch geometry of the strip kernel for one problem.
 struct StripPlan {
     int threads = 0;   // columns of a strip with its halo, one thread each (0: the tile kernels step this problem)
@@ -30,6 +47,14 @@ struct StripPlan {
     int nstrips = 0;
     int ctas = 0;      // CTAs that run at once
 };
+// Rectangles of the FP64 kernel of small grids.
+struct PatchPlan {
+    int tx = 0, ty = 0;   // cells (0: the strip kernel steps this problem)
+    size_t smem = 0;
+};
+cudaError_t patch_plan(bool coupled, bool wally, int nx, int ny, int strip_rows, PatchPlan *out);
+cudaError_t launch_patch(const PatchPlan &pl, const StepArgs<double> &a, const StripPhys<double> &sp,
+                         const Phys<double> &ph, bool coupled, bool wally, cudaStream_t st);
 template <typename Real>
 cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out);
 template <typename Real>
@@ -97,6 +122,7 @@ struct dugks_ctx {
     bool tma_ok;
     CUtensorMap tm_state[2], tm_hist[2];
     dugks::StripPlan strip;
+    dugks::PatchPlan patch;
     dugks::StripMaps strip_maps[2];   // of a step from buffer 0 or 1
     dugks::StripPhys<double> spd;
 

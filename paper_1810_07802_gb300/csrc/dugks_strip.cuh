@@ -257,7 +257,8 @@ struct StripPt {
 // e = 6 num + step rho den, 1 / (2 tau_g + step) = rho den / e and tau_g / (2 tau_g + step) = 3 num / e; FP64
 // takes 1 / rho = den e / (rho den e) from the same division.
 template <typename Real, bool COUPLED>
-__device__ __forceinline__ void strip_closures(const StripPhys<Real> &ph, const PointK<Real> &k, StripPt<Real> &s) {
+__device__ __forceinline__ void strip_closures(const StripPhys<Real> &ph, const PointK<Real> &k, StripPt<Real> &s,
+                                               bool swapped = false) {
     const Real phi = s.phi;
     const Real t = phi * (Real(1) - phi);
     s.tn = t * rsqrt_s(s.G.x * s.G.x + (s.G.y * s.G.y + k.eps));
@@ -273,7 +274,7 @@ __device__ __forceinline__ void strip_closures(const StripPhys<Real> &ph, const 
             const Real r = rd * R;
             s.inv = rd * r;
             s.tin = num * r;
-            V2<Real> g = v2(ph.gx, ph.gy);
+            V2<Real> g = swapped ? v2(ph.gy, ph.gx) : v2(ph.gx, ph.gy);
             if (ph.grav_mode) g = vmul(v2(s.rho - ph.rho_ref), g);
             s.F = vfma(v2(M), s.G, g);
         } else {                             // the two rules and both body forces as linear functions of phi
@@ -355,10 +356,11 @@ template <typename T>
 __device__ __forceinline__ T diag2(T v) { return v2(v.x + v.y, v.y - v.x); }
 
 // The face state and the distributions crossing the face (Eq. 28) from psi-bar and the sums of the two cells'
-// fields; XFACE selects the normal.
+// fields; XFACE selects the normal.  swapped: x and y have changed places, the body force follows.
 template <typename Real, bool COUPLED, bool XFACE>
 __device__ __forceinline__ Flux<Real> strip_face(const StripPhys<Real> &ph, const Dirs<Real> &f, const Dirs<Real> &g,
-                                                 const FaceSum<Real> &m, bool wall, V2<Real> uf) {
+                                                 const FaceSum<Real> &m, bool wall, V2<Real> uf,
+                                                 bool swapped = false) {
     const PointK<Real> &k = ph.face;
     StripPt<Real> s;
     const V2<Real> t = vadd(vadd(f.A, f.B), vadd(f.C, f.D));
@@ -367,7 +369,7 @@ __device__ __forceinline__ Flux<Real> strip_face(const StripPhys<Real> &ph, cons
     s.G = m.G;
     s.E = m.E;
     s.L = m.L;
-    strip_closures<Real, COUPLED>(ph, k, s);
+    strip_closures<Real, COUPLED>(ph, k, s, swapped);
     if constexpr (COUPLED) {
         V2<Real> mm;
         Real sn;
@@ -427,6 +429,113 @@ __device__ __forceinline__ void strip_add_flux(Real dt, const Flux<Real> &in, co
         ga += dt * q.x;
         gb -= dt * q.y;
     }
+}
+
+// Are all three finite (0 x is NaN for an infinity or a NaN)?  FP64 looks at the exponents and signs with integer
+// instructions, which its pipe does not see.
+__device__ __forceinline__ bool all_finite(float a, float b, float c) { return a * 0.0f + b * 0.0f + c * 0.0f == 0.0f; }
+__device__ __forceinline__ bool positive(float a) { return a > 0.0f; }
+__device__ __forceinline__ int hi_word(double v) {
+#ifdef __CUDA_ARCH__
+    return __double2hiint(v);
+#else
+    return 0;
+#endif
+}
+__device__ __forceinline__ bool all_finite(double a, double b, double c) {
+    const int m = 0x7ff00000;
+    return (hi_word(a) & m) != m && (hi_word(b) & m) != m && (hi_word(c) & m) != m;
+}
+__device__ __forceinline__ bool positive(double a) {   // down to 2^-1042
+    return hi_word(a) > 0 && hi_word(a) <= 0x7ff00000;
+}
+
+template <typename Real, bool COUPLED>
+__device__ __forceinline__ V2<Real> strip_velocity(const StepArgs<Real> &a, const Phys<Real> &ph, Real x, Real y,
+                                                   double t) {
+    V2<Real> u = v2(Real(0));
+    if constexpr (!COUPLED) prescribed_velocity(ph, x, y, t, u.x, u.y);
+    return u;
+}
+
+// One cell (Eqs. 29-33) from phi' of three rows, its distributions and history: its record, psi~+ of every direction
+// and the new phi u; u: the velocity of the Allen-Cahn-only model.  Returns status bits.
+template <typename Real, bool COUPLED>
+__device__ __forceinline__ unsigned strip_cell(const StripPhys<Real> &ph, const PhiRow<Real> &pm, const PhiRow<Real> &pc,
+                                               const PhiRow<Real> &pn, const Dirs<Real> &d, Real d0, const Dirs<Real> &dg,
+                                               Real d0g, V2<Real> hist, bool first, V2<Real> u, CellRec<Real, COUPLED> &nr,
+                                               Dirs<Real> &tf, Dirs<Real> &tg, Real &t0f, Real &t0g, V2<Real> &pu) {
+    const PointK<Real> &k = ph.cell;
+    StripPt<Real> s;
+    s.sphi = pc.p;
+    s.phi = ph.phi_ref + pc.p;
+    s.G = v2(Real(4) * pc.d + (pn.d + pm.d), Real(4) * (pn.p - pm.p) + (pn.s - pm.s));
+    s.L = Real(4) * (pc.s + (pn.p + pm.p)) + ((pn.s + pm.s) - Real(20) * pc.p);
+    strip_closures<Real, COUPLED>(ph, k, s);
+    if constexpr (COUPLED) {
+        V2<Real> m;
+        Real sn;
+        strip_moments(dg, m, sn);
+        strip_velocity_pressure(k, m, sn, s);
+    } else {
+        s.u = u;
+    }
+    pu = vmul(v2(s.phi), s.u);
+    s.E = vsub(pu, hist);
+    if (first) s.E = v2(Real(0));
+    nr.G = s.G;
+    nr.E = s.E;
+    nr.L = s.L;
+    const Real k43 = Real(4.0 / 3.0);
+    {   // f: psi-bar-plus = d + e with e = pf_b f_eq + pf_c S - pf_b d, psi~+ = d + 4/3 e; the rest
+        // direction takes minus the sum of the others' e (all nine add up to zero)
+        Real P;
+        V2<Real> V;
+        strip_f_lin(k, s, pu, P, V);
+        const V2<Real> dv = diag2(V), nb = v2(ph.nb), four = v2(Real(4));
+        const V2<Real> eA = vfma(four, vadd(v2(P), V), vmul(nb, d.A));
+        const V2<Real> eB = vfma(four, vsub(v2(P), V), vmul(nb, d.B));
+        const V2<Real> eC = vfma(nb, d.C, vadd(v2(P), dv));
+        const V2<Real> eD = vfma(nb, d.D, vsub(v2(P), dv));
+        nr.f.A = vadd(d.A, eA);
+        nr.f.B = vadd(d.B, eB);
+        nr.f.C = vadd(d.C, eC);
+        nr.f.D = vadd(d.D, eD);
+        tf.A = vfma(v2(k43), eA, d.A);
+        tf.B = vfma(v2(k43), eB, d.B);
+        tf.C = vfma(v2(k43), eC, d.C);
+        tf.D = vfma(v2(k43), eD, d.D);
+        const V2<Real> e4 = vadd(vadd(eC, eD), vadd(eA, eB));
+        const Real e0 = -(e4.x + e4.y);
+        nr.f0 = d0 + e0;
+        t0f = d0 + k43 * e0;
+    }
+    if constexpr (COUPLED) {
+        const GTerms<Real> t = strip_g_terms(k, s);
+        const Real cb = Real(-36) * t.cb;
+        const V2<Real> nb = v2(cb), four = v2(Real(4));
+        V2<Real> E, O;
+        strip_g_eo(t.o, t.b, t.ec, t, E, O);
+        const V2<Real> eA = vfma(four, vadd(E, O), vmul(nb, dg.A));
+        const V2<Real> eB = vfma(four, vsub(E, O), vmul(nb, dg.B));
+        strip_g_eo(diag2(t.o), diag2(t.b), diag2(t.ec), t, E, O);
+        const V2<Real> eC = vfma(nb, dg.C, vadd(E, O));
+        const V2<Real> eD = vfma(nb, dg.D, vsub(E, O));
+        nr.g.A = vadd(dg.A, eA);
+        nr.g.B = vadd(dg.B, eB);
+        nr.g.C = vadd(dg.C, eC);
+        nr.g.D = vadd(dg.D, eD);
+        tg.A = vfma(v2(k43), eA, dg.A);
+        tg.B = vfma(v2(k43), eB, dg.B);
+        tg.C = vfma(v2(k43), eC, dg.C);
+        tg.D = vfma(v2(k43), eD, dg.D);
+        const Real e0 = cb * d0g + (Real(16) * (t.base + t.q0 * t.c0) - Real(36) * t.P);
+        t0g = d0g + k43 * e0;
+    }
+    const bool bad = !all_finite(s.phi, s.u.x, s.u.y);
+    bool nonphys = false;
+    if constexpr (COUPLED) nonphys = !positive(s.rho) || !positive(s.lin);
+    return (bad ? STATUS_NONFINITE : 0u) | (nonphys ? STATUS_NONPHYSICAL : 0u);
 }
 
 // Central reconstruction (Eq. 27) of one model, v = (1/2 + h c_n) a + (1/2 - h c_n) b - h c_t s_t between the
@@ -523,25 +632,6 @@ __device__ __forceinline__ Dirs<Real> strip_wall(const Real *row, const Real *in
     return o;
 }
 
-// Are all three finite (0 x is NaN for an infinity or a NaN)?  FP64 looks at the exponents and signs with integer
-// instructions, which its pipe does not see.
-__device__ __forceinline__ bool all_finite(float a, float b, float c) { return a * 0.0f + b * 0.0f + c * 0.0f == 0.0f; }
-__device__ __forceinline__ bool positive(float a) { return a > 0.0f; }
-__device__ __forceinline__ int hi_word(double v) {
-#ifdef __CUDA_ARCH__
-    return __double2hiint(v);
-#else
-    return 0;
-#endif
-}
-__device__ __forceinline__ bool all_finite(double a, double b, double c) {
-    const int m = 0x7ff00000;
-    return (hi_word(a) & m) != m && (hi_word(b) & m) != m && (hi_word(c) & m) != m;
-}
-__device__ __forceinline__ bool positive(double a) {   // down to 2^-1042
-    return hi_word(a) > 0 && hi_word(a) <= 0x7ff00000;
-}
-
 // cp.async of one element (4 or 8 bytes).
 __device__ __forceinline__ void cp_async_elt(float *dst, const float *src) {
 #ifdef __CUDA_ARCH__
@@ -557,14 +647,6 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *bar) {
 #ifdef __CUDA_ARCH__
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 #endif
-}
-
-template <typename Real, bool COUPLED>
-__device__ __forceinline__ V2<Real> strip_velocity(const StepArgs<Real> &a, const Phys<Real> &ph, Real x, Real y,
-                                                   double t) {
-    V2<Real> u = v2(Real(0));
-    if constexpr (!COUPLED) prescribed_velocity(ph, x, y, t, u.x, u.y);
-    return u;
 }
 
 // Both loads of a staged row, by the thread whose `p` is set (predicated: no branch).
@@ -769,87 +851,33 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
         if (row_in) {
             // ---- the cell of row r ----
             const Real *c = col + cslot * SLOT;
-            const PointK<Real> &k = ph.cell;
-            StripPt<Real> s;
-            s.sphi = pc.p;
-            s.phi = ph.phi_ref + pc.p;
-            s.G = v2(Real(4) * pc.d + (pn.d + pm.d), Real(4) * (pn.p - pm.p) + (pn.s - pm.s));
-            s.L = Real(4) * (pc.s + (pn.p + pm.p)) + ((pn.s + pm.s) - Real(20) * pc.p);
-            strip_closures<Real, COUPLED>(ph, k, s);
-            Dirs<Real> dg;
-            const int yw = WALLY ? r : (r < 0 ? r + ny : (r >= ny ? r - ny : r));
+            Dirs<Real> df, dg;
+            Real d0g = Real(0);
+            df.A = v2(c[1 * BW], c[3 * BW]);
+            df.B = v2(c[5 * BW], c[7 * BW]);
+            df.C = v2(c[2 * BW], c[4 * BW]);
+            df.D = v2(c[6 * BW], c[8 * BW]);
+            V2<Real> u = v2(Real(0));
             if constexpr (COUPLED) {
                 dg.A = v2(c[10 * BW], c[12 * BW]);
                 dg.B = v2(c[14 * BW], c[16 * BW]);
                 dg.C = v2(c[11 * BW], c[13 * BW]);
                 dg.D = v2(c[15 * BW], c[17 * BW]);
-                V2<Real> m;
-                Real sn;
-                strip_moments(dg, m, sn);
-                strip_velocity_pressure(k, m, sn, s);
-            } else if (ph.vel_kind == 0) {
-                s.u = v2(ph.u0x, ph.u0y);
-            } else if (ph.vel_kind == 4) {
-                const long long gv = (long long)yw * a.pitch + xw;
-                s.u = v2(a.vel[gv], a.vel[a.plane + gv]);
+                d0g = c[9 * BW];
             } else {
-                s.u = strip_velocity<Real, COUPLED>(a, pv, Real(xw) + Real(0.5), Real(yw) + Real(0.5), a.t_n);
+                const int yw = WALLY ? r : (r < 0 ? r + ny : (r >= ny ? r - ny : r));
+                if (ph.vel_kind == 0) {
+                    u = v2(ph.u0x, ph.u0y);
+                } else if (ph.vel_kind == 4) {
+                    const long long gv = (long long)yw * a.pitch + xw;
+                    u = v2(a.vel[gv], a.vel[a.plane + gv]);
+                } else {
+                    u = strip_velocity<Real, COUPLED>(a, pv, Real(xw) + Real(0.5), Real(yw) + Real(0.5), a.t_n);
+                }
             }
-            npu = vmul(v2(s.phi), s.u);
-            s.E = vsub(npu, v2(c[HO], c[HO + BW]));
-            if (a.first_step) s.E = v2(Real(0));
-            nr.G = s.G;
-            nr.E = s.E;
-            nr.L = s.L;
-            const Real k43 = Real(4.0 / 3.0);
-            {   // f: psi-bar-plus = d + e with e = pf_b f_eq + pf_c S - pf_b d, psi~+ = d + 4/3 e; the rest
-                // direction takes minus the sum of the others' e (all nine add up to zero)
-                Real P;
-                V2<Real> V;
-                strip_f_lin(k, s, npu, P, V);
-                const V2<Real> dv = diag2(V), nb = v2(ph.nb), four = v2(Real(4));
-                const V2<Real> dA = v2(c[1 * BW], c[3 * BW]), dB = v2(c[5 * BW], c[7 * BW]);
-                const V2<Real> dC = v2(c[2 * BW], c[4 * BW]), dD = v2(c[6 * BW], c[8 * BW]);
-                const V2<Real> eA = vfma(four, vadd(v2(P), V), vmul(nb, dA));
-                const V2<Real> eB = vfma(four, vsub(v2(P), V), vmul(nb, dB));
-                const V2<Real> eC = vfma(nb, dC, vadd(v2(P), dv));
-                const V2<Real> eD = vfma(nb, dD, vsub(v2(P), dv));
-                nr.f.A = vadd(dA, eA);
-                nr.f.B = vadd(dB, eB);
-                nr.f.C = vadd(dC, eC);
-                nr.f.D = vadd(dD, eD);
-                ntf.A = vfma(v2(k43), eA, dA);
-                ntf.B = vfma(v2(k43), eB, dB);
-                ntf.C = vfma(v2(k43), eC, dC);
-                ntf.D = vfma(v2(k43), eD, dD);
-                const V2<Real> e4 = vadd(vadd(eC, eD), vadd(eA, eB));
-                const Real e0 = -(e4.x + e4.y), d0 = c[0];
-                nr.f0 = d0 + e0;
-                n0f = d0 + k43 * e0;
-            }
-            if constexpr (COUPLED) {
-                const GTerms<Real> t = strip_g_terms(k, s);
-                const Real cb = Real(-36) * t.cb;
-                const V2<Real> nb = v2(cb), four = v2(Real(4));
-                V2<Real> E, O;
-                strip_g_eo(t.o, t.b, t.ec, t, E, O);
-                const V2<Real> eA = vfma(four, vadd(E, O), vmul(nb, dg.A));
-                const V2<Real> eB = vfma(four, vsub(E, O), vmul(nb, dg.B));
-                strip_g_eo(diag2(t.o), diag2(t.b), diag2(t.ec), t, E, O);
-                const V2<Real> eC = vfma(nb, dg.C, vadd(E, O));
-                const V2<Real> eD = vfma(nb, dg.D, vsub(E, O));
-                nr.g.A = vadd(dg.A, eA);
-                nr.g.B = vadd(dg.B, eB);
-                nr.g.C = vadd(dg.C, eC);
-                nr.g.D = vadd(dg.D, eD);
-                ntg.A = vfma(v2(k43), eA, dg.A);
-                ntg.B = vfma(v2(k43), eB, dg.B);
-                ntg.C = vfma(v2(k43), eC, dg.C);
-                ntg.D = vfma(v2(k43), eD, dg.D);
-                const Real d0 = c[9 * BW];
-                const Real e0 = cb * d0 + (Real(16) * (t.base + t.q0 * t.c0) - Real(36) * t.P);
-                n0g = d0 + k43 * e0;
-            }
+            const unsigned bad = strip_cell<Real, COUPLED>(ph, pm, pc, pn, df, c[0], dg, d0g, v2(c[HO], c[HO + BW]),
+                                                           a.first_step != 0, u, nr, ntf, ntg, n0f, n0g, npu);
+            if (bad && mine && r >= ya && r < yb) atomicOr(a.status, bad);
             if constexpr (!SHF) {
                 st_pairs(rec + 4 + gCDf, nr.f.C, nr.f.D);
                 st_pairs(rec + 4 + gABf, nr.f.A, nr.f.B);
@@ -859,13 +887,6 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
             if constexpr (COUPLED && !SHF) {
                 st_pairs(rec + 4 + gCDg, nr.g.C, nr.g.D);
                 st_pairs(rec + 4 + gABg, nr.g.A, nr.g.B);
-            }
-            if (mine && r >= ya && r < yb) {
-                const bool bad = !all_finite(s.phi, s.u.x, s.u.y);
-                bool nonphys = false;
-                if constexpr (COUPLED) nonphys = !positive(s.rho) || !positive(s.lin);
-                if (bad || nonphys)
-                    atomicOr(a.status, (bad ? STATUS_NONFINITE : 0u) | (nonphys ? STATUS_NONPHYSICAL : 0u));
             }
         }
         __syncwarp();

@@ -23,13 +23,19 @@ cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out)
     return with_strip(coupled, wally, [&](auto c, auto wl) {
         constexpr bool C = decltype(c)::value, W = decltype(wl)::value;
         using S = StripShape<Real, C, strip_shuffles<Real, W>()>;
-        auto *k = strip_step_kernel<Real, C, W>;
         constexpr size_t bytes = S::smem_bytes(kStripLanes, W);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(strip_batch_kernel<Real, C, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        static OncePerDevice<int> resident;   // CTAs that fit on an SM
         int per_sm = 0;
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kStripLanes, bytes);
+        const cudaError_t e = resident.get(dev, &per_sm, [&](int *out) {
+            cudaError_t r = cudaFuncSetAttribute(strip_step_kernel<Real, C, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)bytes);
+            if (r == cudaSuccess)
+                r = cudaFuncSetAttribute(strip_batch_kernel<Real, C, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)bytes);
+            if (r == cudaSuccess)
+                r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, strip_step_kernel<Real, C, W>, kStripLanes, bytes);
+            return r;
+        });
         if (e != cudaSuccess) return e;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         const int own = S::own(kStripLanes);
