@@ -22,25 +22,18 @@
 
 namespace dugks {
 
-// ---- pairs of values: packed FP32 instructions, plain FP64 ones ----
+// ---- pairs of FP64 values ----
 template <typename Real> struct Pair;
-template <> struct Pair<float> { using T = float2; };
 template <> struct Pair<double> { using T = double2; };
 template <typename Real> using V2 = typename Pair<Real>::T;
 
-__device__ __forceinline__ float2 v2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 v2(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 v2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ double2 v2(double a) { return make_double2(a, a); }
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ double2 vfma(double2 a, double2 b, double2 c) {
     return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
 }
-__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ double2 vmul(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ double2 vadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.0f, -1.0f), b, a); }
 __device__ __forceinline__ double2 vsub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
 // Directions in pairs: A = (1, 3) along +x, +y; B = (5, 7) their opposites; C = (2, 4) the diagonals with
@@ -144,8 +137,6 @@ template <typename Real>
 struct StripPhys {
     PointK<Real> cell, face;
     Real rho_l, drho, visc_a, visc_b, gx, gy, rho_ref, phi_ref, u0x, u0y;
-    Real num_a, num_b, den_a, den_b;   // 6 num and den as linear functions of phi
-    Real ga_x, ga_y, gb_x, gb_y;       // G as a linear function of phi
     Real nb, ff_a;         // -pf_b, ff_a
     Real cp, cm, h2, ht;   // 1/2 + h, 1/2 - h, 2 h, h / 4
     Real dt, h;
@@ -168,7 +159,7 @@ inline StripPhys<Real> strip_phys(const Phys<double> &p) {
         k.kN = Real(c2 * p.theta_k / 36.0);
         k.kD = Real(3.0 * c2 * p.inv_dt / (36.0 * sum));
         k.kb = Real(g / 36.0);
-        k.kc = Real((sizeof(Real) == 8 ? 3.0 : 0.5) * g / 36.0);
+        k.kc = Real(3.0 * g / 36.0);
         return k;
     };
     o.cell = point(1.0, p.pf_b, p.pf_c, p.dt, 3.0 * p.h);
@@ -183,16 +174,6 @@ inline StripPhys<Real> strip_phys(const Phys<double> &p) {
     o.phi_ref = Real(p.phi_ref);
     o.u0x = Real(p.u0x);
     o.u0y = Real(p.u0y);
-    const bool lin = p.visc_linear;
-    o.num_a = Real(lin ? 6.0 * p.visc_a : 0.0);
-    o.num_b = Real(lin ? 6.0 * p.visc_b : 6.0);
-    o.den_a = Real(lin ? 0.0 : p.visc_a);
-    o.den_b = Real(lin ? 1.0 : p.visc_b);
-    const double ga = p.grav_mode ? p.drho : 0.0, gb = p.grav_mode ? p.rho_l - p.rho_ref : 1.0;
-    o.ga_x = Real(ga * p.gx);
-    o.ga_y = Real(ga * p.gy);
-    o.gb_x = Real(gb * p.gx);
-    o.gb_y = Real(gb * p.gy);
     o.nb = Real(-p.pf_b);
     o.ff_a = Real(p.ff_a);
     o.cp = Real(0.5 + p.h);
@@ -207,21 +188,6 @@ inline StripPhys<Real> strip_phys(const Phys<double> &p) {
     return o;
 }
 
-// Hardware reciprocal and reciprocal square root (FP32: one instruction, arguments far from the denormals).
-__device__ __forceinline__ float rcp_s(float x) {
-    float y = x;
-#ifdef __CUDA_ARCH__
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-#endif
-    return y;
-}
-__device__ __forceinline__ float rsqrt_s(float x) {
-    float y = x;
-#ifdef __CUDA_ARCH__
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-#endif
-    return y;
-}
 // FP64: the hardware's 20-bit seed refined once at third order: with e = 1 - x y the series 1 / x = y (1 + e + e^2 +
 // ...), with e = 1 - x y^2 the series 1 / sqrt(x) = y (1 + e / 2 + 3 e^2 / 8 + ...); what is left is of order e^3.
 __device__ __forceinline__ double rcp_s(double x) {
@@ -247,15 +213,15 @@ struct StripPt {
     Real sphi, phi;               // phi - phi_ref, phi
     V2<Real> G, E;
     Real L, rho, irho, lin;
-    Real inv, tin;                // 1 / (2 tau_g + step), tau_g / (3 (2 tau_g + step)) (FP32: 6 times that)
+    Real inv, tin;                // 1 / (2 tau_g + step), tau_g / (3 (2 tau_g + step))
     V2<Real> F, u;
     Real tn;                      // phi (1 - phi) / |G|
     Real Q, usq;                  // p' = 0.6 Q; |u|^2
 };
 
 // Closures of Eqs. 3-4, 6, 9-10, 34-36.  With mu = num / den (linear rule lin / 1, reciprocal rule 1 / lin) and
-// e = 6 num + step rho den, 1 / (2 tau_g + step) = rho den / e and tau_g / (2 tau_g + step) = 3 num / e; FP64
-// takes 1 / rho = den e / (rho den e) from the same division.
+// e = 6 num + step rho den, 1 / (2 tau_g + step) = rho den / e and tau_g / (2 tau_g + step) = 3 num / e;
+// 1 / rho = den e / (rho den e) comes from the same reciprocal.
 template <typename Real, bool COUPLED>
 __device__ __forceinline__ void strip_closures(const StripPhys<Real> &ph, const PointK<Real> &k, StripPt<Real> &s,
                                                bool swapped = false) {
@@ -265,27 +231,17 @@ __device__ __forceinline__ void strip_closures(const StripPhys<Real> &ph, const 
     if constexpr (COUPLED) {
         s.rho = ph.rho_l + ph.drho * phi;
         const Real M = k.kappa * s.L + (k.beta * t) * (phi - Real(0.5));
-        if constexpr (sizeof(Real) == 8) {   // uniform branches cost an FP64 step nothing
-            s.lin = ph.visc_a * phi + ph.visc_b;
-            const Real num = ph.visc_linear ? s.lin : Real(1), den = ph.visc_linear ? Real(1) : s.lin;
-            const Real rd = s.rho * den, e = k.step * rd + Real(6) * num;
-            const Real R = rcp_s(rd * e);
-            s.irho = den * (e * R);
-            const Real r = rd * R;
-            s.inv = rd * r;
-            s.tin = num * r;
-            V2<Real> g = swapped ? v2(ph.gy, ph.gx) : v2(ph.gx, ph.gy);
-            if (ph.grav_mode) g = vmul(v2(s.rho - ph.rho_ref), g);
-            s.F = vfma(v2(M), s.G, g);
-        } else {                             // the two rules and both body forces as linear functions of phi
-            const Real num = ph.num_a * phi + ph.num_b, den = ph.den_a * phi + ph.den_b;
-            s.lin = num * den;
-            const Real rd = s.rho * den, R = rcp_s(k.step * rd + num);
-            s.irho = rcp_s(s.rho);
-            s.inv = rd * R;
-            s.tin = num * R;                 // 6 tau_g / (3 (2 tau_g + step))
-            s.F = vfma(v2(M), s.G, vfma(v2(phi), v2(ph.ga_x, ph.ga_y), v2(ph.gb_x, ph.gb_y)));
-        }
+        s.lin = ph.visc_a * phi + ph.visc_b;
+        const Real num = ph.visc_linear ? s.lin : Real(1), den = ph.visc_linear ? Real(1) : s.lin;
+        const Real rd = s.rho * den, e = k.step * rd + Real(6) * num;
+        const Real R = rcp_s(rd * e);
+        s.irho = den * (e * R);
+        const Real r = rd * R;
+        s.inv = rd * r;
+        s.tin = num * r;
+        V2<Real> g = swapped ? v2(ph.gy, ph.gx) : v2(ph.gx, ph.gy);
+        if (ph.grav_mode) g = vmul(v2(s.rho - ph.rho_ref), g);
+        s.F = vfma(v2(M), s.G, g);
     }
 }
 
@@ -396,7 +352,7 @@ __device__ __forceinline__ Flux<Real> strip_face(const StripPhys<Real> &ph, cons
         o.fn = vfma(v2(Real(4)), v2(P + n, P - n), vmul(a, XFACE ? v2(f.A.x, f.B.x) : v2(f.A.y, f.B.y)));
     }
     if constexpr (COUPLED) {
-        const V2<Real> ga = v2(sizeof(Real) == 8 ? Real(6) * s.tin : s.tin);   // 2 tau_g / (2 tau_g + h)
+        const V2<Real> ga = v2(Real(6) * s.tin);   // 2 tau_g / (2 tau_g + h)
         const GTerms<Real> c = strip_g_terms(k, s);
         V2<Real> E, O;
         strip_g_eo(diag2(c.o), diag2(c.b), diag2(c.ec), c, E, O);
@@ -434,7 +390,6 @@ __device__ __forceinline__ void strip_add_flux(Real dt, const Flux<Real> &in, co
 // Are all three finite (0 x is NaN for an infinity or a NaN)?  FP64 looks at the exponents and signs with integer
 // instructions, which its pipe does not see.
 __device__ __forceinline__ bool all_finite(float a, float b, float c) { return a * 0.0f + b * 0.0f + c * 0.0f == 0.0f; }
-__device__ __forceinline__ bool positive(float a) { return a > 0.0f; }
 __device__ __forceinline__ int hi_word(double v) {
 #ifdef __CUDA_ARCH__
     return __double2hiint(v);
