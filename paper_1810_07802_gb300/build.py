@@ -15,7 +15,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB_NAME = "libdugks_gb300.so"
 LIB_PATH = os.path.join(BUILD_DIR, LIB_NAME)
 SOURCES = ["dugks_capi.cu", "dugks_fp64.cu", "dugks_fp32.cu", "dugks_strip_fp64.cu",
-           "dugks_strip_fp32.cu", "dugks_patch.cu", "dugks_static.cu", "dugks_batch.cu"]
+           "dugks_strip_fp32.cu", "dugks_patch.cu", "dugks_strip_upwind.cu", "dugks_static.cu", "dugks_batch.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

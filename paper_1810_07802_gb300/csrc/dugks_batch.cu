@@ -114,7 +114,7 @@ struct dugks_batch_ctx {
             g.size.clear();
             ph.clear();
             for (dugks_ctx *c : members)
-                if (c->strip.threads && c->fp32 == g.fp32 && c->coupled == g.coupled && c->wally == g.wally &&
+                if (c->strip.threads && !c->upw && c->fp32 == g.fp32 && c->coupled == g.coupled && c->wally == g.wally &&
                     member_tiles(c) < kSoloTiles) {
                     g.members.push_back(c);
                     g.size.push_back(make_int2(c->strip.nstrips, c->P.ny));
@@ -189,7 +189,7 @@ struct dugks_batch_ctx {
                 g.members.clear();
                 for (dugks_ctx *c : members)
                     if (c->fp32 == g.fp32 && c->coupled == g.coupled && c->wally == g.wally && c->tile == g.tile &&
-                        c->upw == g.upw && !c->strip.threads && member_tiles(c) < kSoloTiles)
+                        c->upw == g.upw && (c->upw || !c->strip.threads) && member_tiles(c) < kSoloTiles)
                         g.members.push_back(c);
                 grouped = grouped || !g.members.empty();
                 const int tx = g.fp32 ? dugks::tile_dim<float>(g.tile, 0) : dugks::tile_dim<double>(g.tile, 0);

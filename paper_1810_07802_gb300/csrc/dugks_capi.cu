@@ -103,7 +103,10 @@ cudaError_t step_on(dugks_ctx *c, long long nsteps, cudaStream_t st) {
         if (c->patch.tx) {
             e = launch_patch(c->patch, c->step_args<double>(), c->spd, c->phd, c->coupled, c->wally, st);
         } else if (c->strip.threads) {
-            if (c->fp32)
+            if (c->upw)
+                e = launch_strip_upwind(c->strip, c->strip_maps[c->cur], c->step_args<float>(), c->phf, c->coupled, c->wally,
+                                        st);
+            else if (c->fp32)
                 e = launch_strip<float>(c->strip, c->strip_maps[c->cur], c->step_args<float>(), c->phf, c->phf, c->coupled,
                                         c->wally, st);
             else
@@ -398,9 +401,10 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
                                                   L.pitch, 2, tx + 8, box_rows);
         }
     }
-    if (params->tile_shape == 0 && !c->upw) {
-        cudaError_t es = c->fp32 ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
-                                       : dugks::strip_plan<double>(c->coupled, c->wally, params->nx, params->ny, &c->strip);
+    if (params->tile_shape == 0 && (c->fp32 || !c->upw)) {
+        cudaError_t es = c->upw    ? dugks::strip_upwind_plan(c->coupled, c->wally, params->nx, params->ny, &c->strip)
+                         : c->fp32 ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
+                                   : dugks::strip_plan<double>(c->coupled, c->wally, params->nx, params->ny, &c->strip);
         if (es == cudaSuccess && !c->fp32)
             es = dugks::patch_plan(c->coupled, c->wally, params->nx, params->ny, c->strip.rows, &c->patch);
         if (es != cudaSuccess) {
@@ -417,6 +421,7 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
             };
             map(&m.src_state, c->state(b), L.nq, c->strip.box);
             map(&m.src_hist, c->hist(b), 2, c->strip.box);
+            if (c->upw) continue;   // its rows leave by plain stores
             map(&m.dst_state, c->state(b ^ 1), L.nq, c->strip.own);
             map(&m.dst_hist, c->hist(b ^ 1), 2, c->strip.own);
         }

@@ -60,6 +60,9 @@ cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out)
 template <typename Real>
 cudaError_t launch_strip(const StripPlan &pl, const StripMaps &tm, const StepArgs<Real> &a, const typename StripConst<Real>::T &sp,
                          const Phys<Real> &ph, bool coupled, bool wally, cudaStream_t st);
+cudaError_t strip_upwind_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out);
+cudaError_t launch_strip_upwind(const StripPlan &pl, const StripMaps &tm, const StepArgs<float> &a, const Phys<float> &ph,
+                                bool coupled, bool wally, cudaStream_t st);
 template <typename Real>
 cudaError_t strip_group_rows(bool coupled, bool wally, const int2 *members, int n, int *rows);
 template <typename Real>

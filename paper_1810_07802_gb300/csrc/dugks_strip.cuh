@@ -1229,6 +1229,91 @@ __device__ __forceinline__ void wall32(const float2 c[4], const float2 e[4], con
     if (rest) o0 = out[0];
 }
 
+// One cell: the operations of cell_item.  s holds grad phi and lap phi, c points at the cell's column of the staged
+// row (planes bw apart, the history at ho), p = phi'.  Returns the record; psi~+ (rest directions in t0), phi u.
+template <bool COUPLED>
+__device__ __forceinline__ Rec32 cell32(const Phys<float> &ph, const StepArgs<float> &a, Pt<float> &s, const float *c, int bw,
+                                        int ho, float p, int xw, int yw, float2 tf[4], float2 tg[4], float2 &t0, float2 &pu,
+                                        bool own) {
+    Rec32 nr;
+                s.phi = ph.phi_ref + p;
+                closures<float, COUPLED>(ph, s, ph.dt);
+                float2 dg[4];
+                if (COUPLED) {
+    #pragma unroll
+                    for (int q = 0; q < 4; q++) dg[q] = f2(c[(10 + q) * bw], c[(14 + q) * bw]);
+                    float mx, my, sn;
+                    moments32(dg, mx, my, sn);
+                    velocity_pressure(mx, my, sn, ph.half_dt, s);
+                } else if (ph.vel_kind == 0) {
+                    s.ux = ph.u0x;
+                    s.uy = ph.u0y;
+                } else if (ph.vel_kind == 4) {
+                    const long long gv = (long long)yw * a.pitch + xw;
+                    s.ux = a.vel[gv];
+                    s.uy = a.vel[a.plane + gv];
+                } else {
+                    prescribed_velocity(ph, float(xw) + 0.5f, float(yw) + 0.5f, a.t_n, s.ux, s.uy);
+                }
+                const float phux = s.phi * s.ux, phuy = s.phi * s.uy;
+                if (a.first_step) {
+                    s.Dx = 0.0f;
+                    s.Dy = 0.0f;
+                } else {
+                    s.Dx = mul_sub(s.phi, s.ux, c[ho]) * ph.inv_dt;
+                    s.Dy = mul_sub(s.phi, s.uy, c[ho + bw]) * ph.inv_dt;
+                }
+                pu = f2(phux, phuy);
+                nr.dp = f2(s.dpx, s.dpy);
+                nr.D = f2(s.Dx, s.Dy);
+                nr.lap = s.lap;
+                {
+                    const FLin<float> lf = f_lin(ph, s, ph.pf_b, ph.pf_c);
+                    float2 bsum2 = f2(0.0f);
+                    auto fpair = [&](auto kc) {
+                        constexpr int K = decltype(kc)::value;
+                        const float2 d = f2(c[K * bw], c[(K + 4) * bw]);
+                        const float2 bp = add2(d, fma2(f2(-ph.pf_b), d, f_lin_pair<K>(lf)));
+                        nr.f[K - 1] = bp;
+                        bsum2 = add2(bsum2, bp);
+                        tf[K - 1] = fma2(f2(1.0f / 3.0f), sub2(bp, d), bp);
+                    };
+                    fpair(std::integral_constant<int, 1>{});
+                    fpair(std::integral_constant<int, 2>{});
+                    fpair(std::integral_constant<int, 3>{});
+                    fpair(std::integral_constant<int, 4>{});
+                    const float d = c[0];
+                    const float bp = p - (bsum2.x + bsum2.y);
+                    nr.f0 = bp;
+                    t0.x = bp + (bp - d) * float(1.0 / 3.0);
+                }
+                if (COUPLED) {
+                    const float inv = rcp_r(2.0f * s.taug + ph.dt);
+                    const float cb = 3.0f * ph.h * inv, cc = 3.0f * s.taug * ph.h * inv;
+                    const GLin<float> gl = g_lin(s, cb, cc);
+                    auto gpair = [&](auto kc) {
+                        constexpr int K = decltype(kc)::value;
+                        const float2 d = dg[K - 1];
+                        const float2 bp = add2(d, fma2(f2(-cb), d, g_lin_pair<K>(gl)));
+                        nr.g[K - 1] = bp;
+                        tg[K - 1] = fma2(f2(1.0f / 3.0f), sub2(bp, d), bp);
+                    };
+                    gpair(std::integral_constant<int, 1>{});
+                    gpair(std::integral_constant<int, 2>{});
+                    gpair(std::integral_constant<int, 3>{});
+                    gpair(std::integral_constant<int, 4>{});
+                    const float d = c[9 * bw], bp = d + (g_lin_k(0, gl) - cb * d);
+                    t0.y = bp + (bp - d) * float(1.0 / 3.0);
+                }
+                if (own) {
+                    const bool bad = !all_finite(s.phi, s.ux, s.uy);
+                    const bool nonphys = COUPLED && !(s.rho > 0.0f && s.taug > 0.0f);
+                    if (bad || nonphys)
+                        atomicOr(a.status, (bad ? STATUS_NONFINITE : 0u) | (nonphys ? STATUS_NONPHYSICAL : 0u));
+                }
+    return nr;
+}
+
 template <bool COUPLED, bool WALLY>
 __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArgs<float> &a, const Phys<float> &ph,
                                               int x0, int ya, int yb) {
@@ -1341,81 +1426,10 @@ __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArg
                 s.dpy = (N - Sv) * Real(1.0 / 3.0) + ((NE + NW) - (SE + SW)) * Real(1.0 / 12.0);
                 s.lap = (Real(4) * ((E + Wv) + (N + Sv)) + ((NE + NW) + (SE + SW)) - Real(20) * C) * Real(1.0 / 6.0);
             }
-            s.phi = ph.phi_ref + pc.p;
-            closures<float, COUPLED>(ph, s, ph.dt);
-            float2 dg[4];
-            if (COUPLED) {
-#pragma unroll
-                for (int p = 0; p < 4; p++) dg[p] = f2(c[(10 + p) * BW], c[(14 + p) * BW]);
-                float mx, my, sn;
-                moments32(dg, mx, my, sn);
-                velocity_pressure(mx, my, sn, ph.half_dt, s);
-            } else if (ph.vel_kind == 0) {
-                s.ux = ph.u0x;
-                s.uy = ph.u0y;
-            } else if (ph.vel_kind == 4) {
-                const long long gv = (long long)yw * a.pitch + xw;
-                s.ux = a.vel[gv];
-                s.uy = a.vel[a.plane + gv];
-            } else {
-                prescribed_velocity(ph, float(xw) + 0.5f, float(yw) + 0.5f, a.t_n, s.ux, s.uy);
-            }
-            const float phux = s.phi * s.ux, phuy = s.phi * s.uy;
-            if (a.first_step) {
-                s.Dx = 0.0f;
-                s.Dy = 0.0f;
-            } else {
-                s.Dx = mul_sub(s.phi, s.ux, c[HO]) * ph.inv_dt;
-                s.Dy = mul_sub(s.phi, s.uy, c[HO + BW]) * ph.inv_dt;
-            }
-            npu = f2(phux, phuy);
-            nr.dp = f2(s.dpx, s.dpy);
-            nr.D = f2(s.Dx, s.Dy);
-            nr.lap = s.lap;
-            {
-                const FLin<float> lf = f_lin(ph, s, ph.pf_b, ph.pf_c);
-                float2 bsum2 = f2(0.0f);
-                auto fpair = [&](auto kc) {
-                    constexpr int K = decltype(kc)::value;
-                    const float2 d = f2(c[K * BW], c[(K + 4) * BW]);
-                    const float2 bp = add2(d, fma2(f2(-ph.pf_b), d, f_lin_pair<K>(lf)));
-                    nr.f[K - 1] = bp;
-                    bsum2 = add2(bsum2, bp);
-                    ntf[K - 1] = fma2(f2(1.0f / 3.0f), sub2(bp, d), bp);
-                };
-                fpair(std::integral_constant<int, 1>{});
-                fpair(std::integral_constant<int, 2>{});
-                fpair(std::integral_constant<int, 3>{});
-                fpair(std::integral_constant<int, 4>{});
-                const float d = c[0];
-                const float bp = pc.p - (bsum2.x + bsum2.y);
-                nr.f0 = bp;
-                n0f = bp + (bp - d) * Real(1.0 / 3.0);
-            }
-            if (COUPLED) {
-                const float inv = rcp_r(2.0f * s.taug + ph.dt);
-                const float cb = 3.0f * ph.h * inv, cc = 3.0f * s.taug * ph.h * inv;
-                const GLin<float> gl = g_lin(s, cb, cc);
-                auto gpair = [&](auto kc) {
-                    constexpr int K = decltype(kc)::value;
-                    const float2 d = dg[K - 1];
-                    const float2 bp = add2(d, fma2(f2(-cb), d, g_lin_pair<K>(gl)));
-                    nr.g[K - 1] = bp;
-                    ntg[K - 1] = fma2(f2(1.0f / 3.0f), sub2(bp, d), bp);
-                };
-                gpair(std::integral_constant<int, 1>{});
-                gpair(std::integral_constant<int, 2>{});
-                gpair(std::integral_constant<int, 3>{});
-                gpair(std::integral_constant<int, 4>{});
-                const float d = c[9 * BW], bp = d + (g_lin_k(0, gl) - cb * d);
-                n0g = bp + (bp - d) * Real(1.0 / 3.0);
-            }
-            if (mine && r >= ya && r < yb) {
-                const bool bad = !all_finite(s.phi, s.ux, s.uy);
-                const bool nonphys = COUPLED && !(s.rho > 0.0f && s.taug > 0.0f);
-                if (bad || nonphys)
-                    atomicOr(a.status, (bad ? STATUS_NONFINITE : 0u) | (nonphys ? STATUS_NONPHYSICAL : 0u));
-            }
+            float2 nt0 = f2(0.0f);
+            nr = cell32<COUPLED>(ph, a, s, c, BW, HO, pc.p, xw, yw, ntf, ntg, nt0, npu, mine && r >= ya && r < yb);
+            n0f = nt0.x;
+            n0g = nt0.y;
         }
         __syncwarp();
         load_row(j + 1 + S::S, cslot);   // the slot of row r is free: every lane has read it

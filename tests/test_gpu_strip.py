@@ -63,3 +63,14 @@ def test_large_grids_against_the_tile_kernels(S, precision, nx, ny, model, bc_y)
     cfg = dict(cfg, precision=precision, phi_ref=0.5)
     strip, tile = (stepped(S, dict(cfg, tile_shape=k), f, 3) for k in (0, 1))
     assert np.abs(strip - tile).max() <= (1e-12 if precision == "fp64" else 4e-7) * np.abs(tile).max()
+
+
+@pytest.mark.parametrize("bc_y", ["periodic", "wall"])
+@pytest.mark.parametrize("model", ["coupled", "ac"])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (4, 200), (25, 6), (26, 9), (27, 8), (53, 12), (130, 70), (1003, 777)])
+def test_upwind_strips_against_the_tile_kernels(S, nx, ny, model, bc_y):
+    """The FP32 upwind strips (26 columns of their own, three-row halo) against the tile kernel's slopes."""
+    cfg, f = problem(nx, ny, model, bc_y)
+    cfg = dict(cfg, precision="fp32", phi_ref=0.5, recon="upwind")
+    strip, tile = (stepped(S, dict(cfg, tile_shape=k), f, 3) for k in (0, 1))
+    assert np.abs(strip - tile).max() <= 4e-7 * np.abs(tile).max()
