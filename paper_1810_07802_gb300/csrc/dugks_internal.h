@@ -45,7 +45,8 @@ struct StripPlan {
     int own = 0;       // columns of a finished row
     int rows = 0;      // rows of a chunk
     int nstrips = 0;
-    int ctas = 0;      // CTAs that run at once
+    int max_warps = 1; // warps a scheduler holds at most
+    size_t smem = 0;   // of a CTA
 };
 // Rectangles of the FP64 kernel of small grids.
 struct PatchPlan {

@@ -9,13 +9,12 @@
 // Why a march: a tile of 32 x 8 cells computes a ring of 84 more records and 8 % of its faces twice, holds all of it
 // in shared memory between four CTA barriers, and spends a fifth of its instructions on addresses.  A strip
 // computes 32 records and 64 faces for 28 cells (14 % more than it needs; two record rows more per chunk) and
-// meets no barrier at all.  What bounds it: FP32, issue slots (69 % active with two warps a scheduler; 12 warps an SM need
-// 168 registers and the carried values in shared memory: no faster; any spill doubles the time, the first-level cache being the
-// shared memory); FP64, the FP64 pipe (83 % active).  Wider strips exchange columns through shared memory behind
-// CTA barriers: 64 to 224 columns are 5 to 80 % slower in FP32 and equal in FP64.
+// meets no barrier at all.  What bounds it: FP32, issue slots (any spill doubles the time, the first-level cache being
+// what the shared memory leaves); FP64, the FP64 pipe (83 % active).  Wider strips exchange columns through shared
+// memory behind CTA barriers: 64 to 224 columns are 5 to 80 % slower in FP32 and equal in FP64.
 //
-// Measured, tile kernel -> strip kernel: FP32 2048^2 287 -> 221 us a step, 4096^2 1,150 -> 867, 509 x 387 26.5 -> 16.3,
-// 64^2 10.3 -> 5.8, 256 x 1024 between walls 28.9 -> 21.2; FP64 1024^2 2,464 -> 1,760, 512^2 616 -> 527.
+// Measured, tile kernel -> strip kernel: FP32 2048^2 287 -> 206 us a step, 4096^2 1,150 -> 794, 509 x 387 26.9 -> 16.6,
+// 64^2 10.3 -> 5.0, 256 x 1024 between walls 28.9 -> 21.4; FP64 1024^2 2,464 -> 1,757.
 #pragma once
 
 #include "dugks_device.cuh"
@@ -68,11 +67,24 @@ struct Flux {
 constexpr int kStripLanes = 32;   // columns of a strip with its halo: one warp
 constexpr int kStripCtas = 8;     // CTAs the register allocation leaves room for on an SM: two warps a scheduler
 
-template <typename Real, bool COUPLED, bool SHF>
+// FP32 without walls keeps psi~+ and the south flux of the row below in shared memory (52 values a lane): 156
+// registers instead of 225, three warps a scheduler instead of two (2048^2 212 -> 206 us, 4096^2 829 -> 794).  With
+// walls the top wall's flux stays in registers too and the same cap spills.
+template <typename Real, bool WALLY>
+__host__ __device__ constexpr bool strip_keeps() {
+    return sizeof(Real) == 4 && !WALLY;
+}
+template <typename Real, bool WALLY>
+__host__ __device__ constexpr int strip_ctas() {
+    return strip_keeps<Real, WALLY>() ? 12 : kStripCtas;
+}
+
+template <typename Real, bool COUPLED, bool SHF, bool KEEP>
 struct StripShape {
     static constexpr int HX = 2;                   // phi halo: columns on each side of the strip's own
     static constexpr int NQ = COUPLED ? 18 : 9;
-    static constexpr int S = sizeof(Real) == 4 ? 4 : 3;   // staged rows in flight or in use
+    static constexpr int S = sizeof(Real) == 4 && !KEEP ? 4 : 3;   // staged rows in flight or in use
+    static constexpr int KG = COUPLED ? 13 : 8;    // kept groups of 4 values: psi~+ of two rows, one flux
     static constexpr int AL = 128 / int(sizeof(Real));
     static constexpr int RG = SHF ? 0 : (COUPLED ? 6 : 4);   // record groups of 4 values (exchanged by shuffles: none)
     __host__ __device__ static constexpr int up(int v) { return (v + AL - 1) / AL * AL; }
@@ -82,7 +94,7 @@ struct StripShape {
     __host__ __device__ static constexpr int hist_off(int w) { return up(NQ * box(w)); }
     __host__ __device__ static constexpr int slot(int w) { return hist_off(w) + up(2 * box(w)); }
     __host__ __device__ static constexpr int rec_rows(bool wally) { return wally ? 2 : 1; }
-    // offsets in elements: staged rows, the finished row, records, fluxes, phi row, barriers
+    // offsets in elements: staged rows, the finished row, records, fluxes, phi row or kept values, barriers
     __host__ __device__ static constexpr int off_out(int w) { return S * slot(w); }
     __host__ __device__ static constexpr int out_hist(int w) { return up(NQ * own(w)); }
     __host__ __device__ static constexpr int off_rec(int w) { return off_out(w) + out_hist(w) + up(2 * own(w)); }
@@ -93,7 +105,7 @@ struct StripShape {
     __host__ __device__ static constexpr int off_phi(int w, bool wally) {
         return off_flux(w, wally) + (SHF ? 0 : up((COUPLED ? 12 : 6) * (w + 1) + 4));
     }
-    __host__ __device__ static constexpr int off_bar(int w, bool wally) { return off_phi(w, wally) + (SHF ? 0 : up(w + 2)); }
+    __host__ __device__ static constexpr int off_bar(int w, bool wally) { return off_phi(w, wally) + (SHF ? 0 : up(w + 2)) + (KEEP ? KG * 4 * w : 0); }
     __host__ __device__ static constexpr size_t smem_bytes(int w, bool wally) {
         return size_t(off_bar(w, wally)) * sizeof(Real) + S * 8 + 128;
     }
@@ -685,7 +697,7 @@ template <typename Real, bool COUPLED, bool WALLY>
 __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<Real> &a, const StripPhys<Real> &ph,
                                             const Phys<Real> &pv, int x0, int ya, int yb) {
     constexpr bool SHF = strip_shuffles<Real, WALLY>();
-    using S = StripShape<Real, COUPLED, SHF>;
+    using S = StripShape<Real, COUPLED, SHF, false>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Real *sm = reinterpret_cast<Real *>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
     constexpr int W = kStripLanes;
@@ -1193,6 +1205,12 @@ __device__ __forceinline__ void flux32(float dt, const Flux32 &in, const Flux32 
     }
 }
 
+__device__ __forceinline__ float4 group32(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
+__device__ __forceinline__ void ungroup32(const float4 &v, float2 &a, float2 &b) {
+    a = f2(v.x, v.y);
+    b = f2(v.z, v.w);
+}
+
 // A wall face (R9) from the cell next to the wall, its east and west neighbours and the next cell into the fluid:
 // recon_wall on registers.
 template <bool TOP>
@@ -1318,7 +1336,8 @@ template <bool COUPLED, bool WALLY>
 __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArgs<float> &a, const Phys<float> &ph,
                                               int x0, int ya, int yb) {
     using Real = float;
-    using S = StripShape<float, COUPLED, true>;
+    constexpr bool KEEP = strip_keeps<float, WALLY>();
+    using S = StripShape<float, COUPLED, true, KEEP>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *sm = reinterpret_cast<float *>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
     constexpr int W = kStripLanes;
@@ -1327,6 +1346,7 @@ __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArg
     float *ring = sm;
     float *sout = sm + S::off_out(W);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + S::off_bar(W, WALLY));
+    float4 *keep = reinterpret_cast<float4 *>(sm + S::off_phi(W, WALLY)) + tid;   // this lane's groups, W apart
     const int nx = a.nx, ny = a.ny;
     const int x = x0 - S::HX + tid;
     const int xend = min(x0 + OW, nx);
@@ -1430,6 +1450,17 @@ __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArg
             nr = cell32<COUPLED>(ph, a, s, c, BW, HO, pc.p, xw, yw, ntf, ntg, nt0, npu, mine && r >= ya && r < yb);
             n0f = nt0.x;
             n0g = nt0.y;
+        }
+        constexpr int TG = COUPLED ? 5 : 3;   // groups of one row's psi~+
+        if (KEEP && row_in) {
+            float4 *k = keep + (j & 1) * TG * W;
+            k[0] = group32(ntf[0], ntf[1]);
+            k[W] = group32(ntf[2], ntf[3]);
+            k[2 * W] = group32(f2(n0f, n0g), npu);
+            if (COUPLED) {
+                k[3 * W] = group32(ntg[0], ntg[1]);
+                k[4 * W] = group32(ntg[2], ntg[3]);
+            }
         }
         __syncwarp();
         load_row(j + 1 + S::S, cslot);   // the slot of row r is free: every lane has read it
@@ -1567,6 +1598,24 @@ __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArg
                 xe.f[i] = from_east(xf.f[i]);
                 if (COUPLED) xe.g[i] = from_east(xf.g[i]);
             }
+            if (KEEP) {
+                const float4 *k = keep + ((j - 1) & 1) * TG * W;
+                float2 t0;
+                ungroup32(k[0], tf[0], tf[1]);
+                ungroup32(k[W], tf[2], tf[3]);
+                ungroup32(k[2 * W], t0, pu);
+                t0f = t0.x;
+                t0g = t0.y;
+                if (COUPLED) {
+                    ungroup32(k[3 * W], tg[0], tg[1]);
+                    ungroup32(k[4 * W], tg[2], tg[3]);
+                }
+                k = keep + 2 * TG * W;
+                float2 unused;
+                ungroup32(k[0], yS.f[0], yS.f[1]);
+                ungroup32(k[W], yS.f[2], COUPLED ? yS.g[0] : unused);
+                if (COUPLED) ungroup32(k[2 * W], yS.g[1], yS.g[2]);
+            }
             flux32<COUPLED, true>(ph.dt, xf, xe, tf, tg);
             flux32<COUPLED, false>(ph.dt, yS, yN, tf, tg);
             tma_store_wait_read();   // (only the issuing lane has any)
@@ -1589,15 +1638,24 @@ __device__ __forceinline__ void strip_march32(const StripMaps &tm, const StepArg
                 fence_proxy_async_smem();
             }
         }
-        yS = yN;
+        if (KEEP) {
+            if (j >= 1) {
+                float4 *k = keep + 2 * TG * W;
+                k[0] = group32(yN.f[0], yN.f[1]);
+                k[W] = group32(yN.f[2], COUPLED ? yN.g[0] : f2(0.0f));
+                if (COUPLED) k[2 * W] = group32(yN.g[1], yN.g[2]);
+            }
+        } else {
+            yS = yN;
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            tf[p] = ntf[p];
-            tg[p] = ntg[p];
+            for (int p = 0; p < 4; p++) {
+                tf[p] = ntf[p];
+                tg[p] = ntg[p];
+            }
+            t0f = n0f;
+            t0g = n0g;
+            pu = npu;
         }
-        t0f = n0f;
-        t0g = n0g;
-        pu = npu;
         cur = nr;
         pm = pc;
         pc = pn;
@@ -1625,11 +1683,11 @@ __device__ __forceinline__ void strip_run(const StripMaps &tm, const StepArgs<do
 }
 
 template <typename Real, bool COUPLED, bool WALLY>
-__global__ void __launch_bounds__(kStripLanes, kStripCtas)
+__global__ void __launch_bounds__(kStripLanes, (strip_ctas<Real, WALLY>()))
 strip_step_kernel(const __grid_constant__ StripMaps tm, const __grid_constant__ StepArgs<Real> a,
                   const __grid_constant__ typename StripConst<Real>::T ph, const __grid_constant__ Phys<Real> pv,
                   const __grid_constant__ StripArgs g) {
-    using S = StripShape<Real, COUPLED, strip_shuffles<Real, WALLY>()>;
+    using S = StripShape<Real, COUPLED, strip_shuffles<Real, WALLY>(), strip_keeps<Real, WALLY>()>;
     const int strip = (int)blockIdx.x % g.nstrips, chunk = (int)blockIdx.x / g.nstrips;
     const int ya = chunk * g.rows;
     strip_run<COUPLED, WALLY>(tm, a, ph, pv, strip * S::own(kStripLanes), ya, min(ya + g.rows, a.ny));
@@ -1661,9 +1719,9 @@ struct StripGroup {
 };
 
 template <typename Real, bool COUPLED, bool WALLY>
-__global__ void __launch_bounds__(kStripLanes, kStripCtas)
+__global__ void __launch_bounds__(kStripLanes, (strip_ctas<Real, WALLY>()))
 strip_batch_kernel(const __grid_constant__ StripGroup<Real> g) {
-    using S = StripShape<Real, COUPLED, strip_shuffles<Real, WALLY>()>;
+    using S = StripShape<Real, COUPLED, strip_shuffles<Real, WALLY>(), strip_keeps<Real, WALLY>()>;
     const int b = (int)blockIdx.x;
     int lo = 0, hi = g.n;   // the member whose CTAs hold b
     while (hi - lo > 1) {

@@ -31,8 +31,7 @@ cudaError_t strip_upwind_plan(bool coupled, bool wally, int nx, int ny, StripPla
         out->box = UpwindShape<C>::BW;
         out->own = kUpwindOwn;
         out->nstrips = (nx + kUpwindOwn - 1) / kUpwindOwn;
-        out->ctas = kStripCtas * sms;
-        const long long chunks = out->ctas > out->nstrips ? out->ctas / out->nstrips : 1;
+        const long long ctas = (long long)kStripCtas * sms, chunks = ctas > out->nstrips ? ctas / out->nstrips : 1;
         out->rows = (int)((ny + chunks - 1) / chunks);
         return cudaSuccess;
     });
