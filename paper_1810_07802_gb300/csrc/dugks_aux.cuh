@@ -4,6 +4,7 @@
 #pragma once
 
 #include "dugks_device.cuh"
+#include "dugks_strip.cuh"
 
 namespace dugks {
 
@@ -79,20 +80,47 @@ __global__ void init_kernel(const double *__restrict__ in, Real *__restrict__ st
     hist[plane + g] = Real(s.phi * s.uy);
 }
 
+// A stored value as FP64.  FP32 values are widened by integer instructions: the conversion instruction runs at the
+// FP64 pipe's rate (16 cycles a warp and SM), and 18 of them per cell would be a quarter of the macros' time.  The
+// exponent moves by 1023 - 127, the 23 fraction bits by 29 places; zeros keep their sign, denormals, infinities and NaNs
+// take the instruction.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+#ifdef __CUDA_ARCH__
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) {
+        double w;   // volatile: not to be computed beside the common case
+        asm volatile("cvt.f64.f32 %0, %1;" : "=d"(w) : "f"(v));
+        return w;
+    }
+    const unsigned hi = m == 0u ? b : ((b & 0x80000000u) | ((m >> 3) + 0x38000000u));
+    return __hiloint2double((int)hi, (int)(b << 29));
+#else
+    return double(v);
+#endif
+}
+
 // phi' = sum_i d^f_i per cell, in FP64 (Eq. 31 on deviations).
 template <typename Real>
 __global__ void phi_kernel(FieldArgs<Real> a, double *__restrict__ phid) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= a.nx || y >= a.ny) return;
     const long long g = (long long)y * a.pitch + x;
+    Real d[9];
+#pragma unroll
+    for (int k = 0; k < 9; k++) d[k] = a.state[k * a.plane + g];
     double s = 0.0;
 #pragma unroll
-    for (int k = 0; k < 9; k++) s += double(a.state[k * a.plane + g]);
+    for (int k = 0; k < 9; k++) s += widen(d[k]);
     phid[(long long)y * a.nx + x] = s;
 }
 
 // Cell-centre macros (Eqs. 31-33) in FP64 from phi' and the g deviations.
 // out: phi, p, ux, uy planes of [ny][nx] (a NULL plane is skipped).
+// Bound by the FP64 pipe (85 % active; FP32 1024^2: 149 us, 118 without the pressure, and all of the fields and
+// sums of that grid 558 -> 453).  Of the closures only the density, the force and one reciprocal are formed, the
+// moments leave out the products with zero lattice components, and a NULL p saves the pressure.  The force keeps the
+// operations of `closures`: where a cell is at rest, u is the difference of two nearly equal terms.
 template <typename Real, bool COUPLED, bool WALLY>
 __global__ void macro_kernel(FieldArgs<Real> a, const double *__restrict__ phid, Phys<double> ph,
                              double *__restrict__ ophi, double *__restrict__ op, double *__restrict__ oux,
@@ -100,32 +128,46 @@ __global__ void macro_kernel(FieldArgs<Real> a, const double *__restrict__ phid,
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= a.nx || y >= a.ny) return;
     const long long c = (long long)y * a.nx + x, g = (long long)y * a.pitch + x;
-    Pt<double> s;
-    phi_stencils_global<WALLY>(phid, a.nx, a.ny, x, y, s.dpx, s.dpy, s.lap);
-    s.phi = ph.phi_ref + phid[c];
-    closures<double, COUPLED>(ph, s);
+    const double phi = ph.phi_ref + phid[c];
+    double ux = 0.0, uy = 0.0, pd = 0.0;
     if (COUPLED) {
-        double mx = 0.0, my = 0.0, sn = 0.0;
+        Real v[9];
 #pragma unroll
-        for (int k = 0; k < 9; k++) {
-            const double d = double(a.state[(9 + k) * a.plane + g]);
-            mx += double(cx(k)) * d;
-            my += double(cy(k)) * d;
-            if (k) sn += d;
+        for (int k = 1; k < 9; k++) v[k] = a.state[(9 + k) * a.plane + g];
+        double dpx, dpy, lap;
+        phi_stencils_global<WALLY>(phid, a.nx, a.ny, x, y, dpx, dpy, lap);
+        const double rho = ph.rho_l + ph.drho * phi;
+        const double muphi = ph.beta4 * phi * (phi - 1.0) * (phi - 0.5) - ph.kappa * lap;
+        double Gx = ph.gx, Gy = ph.gy;
+        if (ph.grav_mode) {
+            Gx = (rho - ph.rho_ref) * ph.gx;
+            Gy = (rho - ph.rho_ref) * ph.gy;
         }
-        velocity_pressure(mx, my, sn, ph.half_dt, s);
+        const double Fx = muphi * dpx + Gx, Fy = muphi * dpy + Gy, irho = rcp_s(rho);
+        double d[9];
+#pragma unroll
+        for (int k = 1; k < 9; k++) d[k] = widen(v[k]);
+        const double mx = ((((d[1] + d[2]) - d[4]) - d[5]) - d[6]) + d[8];
+        const double my = ((((d[2] + d[3]) + d[4]) - d[6]) - d[7]) - d[8];
+        ux = (mx + ph.half_dt * Fx) * irho;
+        uy = (my + ph.half_dt * Fy) * irho;
+        if (op) {
+            double sn = d[1];
+#pragma unroll
+            for (int k = 2; k < 9; k++) sn += d[k];
+            pd = 0.6 * (sn + ph.half_dt * (ux * (ph.drho * dpx) + uy * (ph.drho * dpy))
+                        - (2.0 / 3.0) * rho * (ux * ux + uy * uy));
+        }
     } else if (ph.vel_kind == 4) {
-        s.ux = double(a.vel[g]);
-        s.uy = double(a.vel[a.plane + g]);
-        s.pd = 0.0;
+        ux = double(a.vel[g]);
+        uy = double(a.vel[a.plane + g]);
     } else {
-        prescribed_velocity(ph, double(x) + 0.5, double(y) + 0.5, a.t, s.ux, s.uy);
-        s.pd = 0.0;
+        prescribed_velocity(ph, double(x) + 0.5, double(y) + 0.5, a.t, ux, uy);
     }
-    if (ophi) ophi[c] = s.phi;
-    if (op) op[c] = ph.p_ref + s.pd;
-    if (oux) oux[c] = s.ux;
-    if (ouy) ouy[c] = s.uy;
+    if (ophi) ophi[c] = phi;
+    if (op) op[c] = ph.p_ref + pd;
+    if (oux) oux[c] = ux;
+    if (ouy) ouy[c] = uy;
 }
 
 // Absolute FP64 distributions [nq][ny][nx] and history [2][ny][nx].

@@ -48,7 +48,7 @@ __global__ void batch_wait_probe_kernel(unsigned long long budget_ns, const unsi
 // the 2 history planes, elements of T) to or from a contiguous buffer
 // [nq + 2][nrows][nx].  Bound by HBM: one vector of V elements a thread, its
 // place from the block's coordinates (dividing a flat index three times per
-// element made it 315 us for the 20 planes of 2048^2 FP32, 670 MB; now 118).
+// element made it 315 us for the 20 planes of 2048^2 FP32, 670 MB; now 103).
 template <typename T, typename VT>
 __global__ void rows_kernel(T *state, T *hist, int nq, int pitch, long long plane, int nx, int row0, int nrows,
                             T *buf, int to_buf) {
@@ -91,9 +91,9 @@ cudaError_t launch_rows(void *state, void *hist, size_t elt, int nq, int pitch, 
 }
 
 cudaError_t launch_reduce(const double *phi, const double *ux, const double *uy, const double *snap, long long n,
-                          long long sstride, int have_snap, double *partial, double *out, cudaStream_t st) {
-    reduce_partial_kernel<<<RED_BLOCKS, RED_THREADS, 0, st>>>(phi, ux, uy, snap, n, sstride, have_snap, partial);
-    reduce_final_kernel<<<1, 32, 0, st>>>(partial, out);
+                          long long sstride, int have_snap, double *keep, double *partial, double *out, cudaStream_t st) {
+    reduce_partial_kernel<<<RED_BLOCKS, RED_THREADS, 0, st>>>(phi, ux, uy, snap, n, sstride, have_snap, keep, partial);
+    reduce_final_kernel<<<1, 32 * RED_VALS, 0, st>>>(partial, out);
     return cudaGetLastError();
 }
 
@@ -375,6 +375,7 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
     c->status_seen = 0;
     c->phd = make_phys<double>(*params);
     c->phf = make_phys<float>(*params);
+    c->spd = dugks::strip_phys<double>(c->phd);
     if (device_workspace) {
         c->ws = static_cast<unsigned char *>(device_workspace);
         c->owns = false;
@@ -412,7 +413,6 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
             delete c;
             return from_cuda(es);
         }
-        c->spd = dugks::strip_phys<double>(c->phd);
         bool ok = true;
         for (int b = 0; b < 2; b++) {
             dugks::StripMaps &m = c->strip_maps[b];
@@ -496,14 +496,18 @@ dugks_status reduce_sums(dugks_handle c, int32_t row0, int32_t nrows, double *r,
     *filled = 0;
     double *s = c->stage();
     const size_t n = c->L.n, off = (size_t)row0 * c->P.nx, m = (size_t)nrows * c->P.nx;
-    cudaError_t e = run_macros(c, s, s + n, s + 2 * n, s + 3 * n);
+    // the sums need no pressure; over the whole grid the partial sums leave the new snapshot behind as they read
+    const bool whole = m == n;
+    cudaError_t e = run_macros(c, s, nullptr, s + 2 * n, s + 3 * n);
     if (e == cudaSuccess)
         e = dugks::launch_reduce(s + off, s + 2 * n + off, s + 3 * n + off, c->snap() + off, (long long)m,
-                                 (long long)n, c->have_snap, c->partial(), c->redout(), c->st);
+                                 (long long)n, c->have_snap, whole ? c->snap() : nullptr, c->partial(), c->redout(),
+                                 c->st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(r, c->redout(), dugks::RED_VALS * sizeof(double), cudaMemcpyDeviceToHost, c->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->snap(), s, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && !whole)
+        e = cudaMemcpyAsync(c->snap(), s, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
+    if (e == cudaSuccess && !whole)
         e = cudaMemcpyAsync(c->snap() + n, s + 2 * n, 2 * n * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
     if (e != cudaSuccess) return from_cuda(e);
     dugks_status st = sync_status(c);
