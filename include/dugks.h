@@ -91,10 +91,12 @@ typedef struct {
     int32_t bc_y;          /* periodic, or no-slip walls on y = 0 and y = ny       */
     int32_t visc_interp;   /* dugks_visc: 1/mu linear in phi (Eq. 35) or mu (Eq. 36) */
     int32_t gravity_mode;  /* 0: G = (gx, gy); 1: G = (rho - rho_ref)(gx, gy)      */
-    int32_t tile_shape;    /* step-kernel tile: 0 the library default, k >= 1 the
-                              k-th compiled shape of the precision (see
-                              dugks_tile_shapes, dugks_autotune).  Every shape
-                              computes the same scheme                             */
+    int32_t tile_shape;    /* 0: the library's choice of step kernel (one warp
+                              marching up a strip of columns, rectangles for
+                              small or upwind FP64 grids); k >= 1: the tile
+                              kernel of the k-th compiled shape of the precision
+                              (see dugks_tile_shapes, dugks_autotune).  All
+                              compute the same scheme                              */
     double cfl;            /* dt = cfl (Eq. 37 with delta_x = 1, RT = 1/3), > 0    */
     double mobility;       /* M_phi > 0; tau_f = M_phi / RT (Eq. 34)               */
     double width;          /* interface width W > 0 (Eq. 3)                        */
@@ -166,7 +168,7 @@ dugks_status dugks_check_batch_wait(int64_t budget_ns, void *cuda_stream);
 /* Tile shapes the step kernels are compiled for, for one precision: writes
  * up to `cap` (tx, ty) cell counts (tx may be NULL, likewise ty) and returns
  * how many there are (tile_shape k >= 1 selects entry k - 1), or -1 for an
- * unknown precision.  Shape 1 is the library default.  No device work. */
+ * unknown precision.  Shape 1 is the tile kernels' default.  No device work. */
 int32_t dugks_tile_shapes(int32_t precision, int32_t *tx, int32_t *ty, int32_t cap);
 
 /* Autotuner of the step kernel's tile shape for one problem.  For every
@@ -275,7 +277,9 @@ dugks_status dugks_destroy(dugks_handle h);
  * A batch advances every member by the same number of DUGKS steps.  Members
  * are grouped by kernel variant (precision x model x y-boundary x tile shape
  * x reconstruction).  By default each group and step is one grid launch over
- * the group's (problem, tile) items.  In the persistent mode
+ * the group's (problem, strip chunk) or (problem, tile) items.  In the
+ * persistent mode, which concerns the members the tile kernels step (the
+ * others' launches already overlap),
  * (dugks_batch_set_persistent(b, 1)) a group advances up to 16 steps in one
  * launch: CTAs (at most one step's items, at most as many as fit on the GPU)
  * take (step, problem, tile) items from one queue in step order, and a tile

@@ -101,7 +101,7 @@ cudaError_t step_on(dugks_ctx *c, long long nsteps, cudaStream_t st) {
     for (long long n = 0; n < nsteps; n++) {
         cudaError_t e;
         if (c->patch.tx) {
-            e = launch_patch(c->patch, c->step_args<double>(), c->spd, c->phd, c->coupled, c->wally, st);
+            e = launch_patch(c->patch, c->step_args<double>(), c->spd, c->phd, c->coupled, c->wally, c->upw, st);
         } else if (c->strip.threads) {
             if (c->upw)
                 e = launch_strip_upwind(c->strip, c->strip_maps[c->cur], c->step_args<float>(), c->phf, c->coupled, c->wally,
@@ -402,12 +402,13 @@ dugks_status dugks_create(const dugks_params *params, const double *phi0, const 
                                                   L.pitch, 2, tx + 8, box_rows);
         }
     }
-    if (params->tile_shape == 0 && (c->fp32 || !c->upw)) {
-        cudaError_t es = c->upw    ? dugks::strip_upwind_plan(c->coupled, c->wally, params->nx, params->ny, &c->strip)
-                         : c->fp32 ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
-                                   : dugks::strip_plan<double>(c->coupled, c->wally, params->nx, params->ny, &c->strip);
+    if (params->tile_shape == 0) {
+        cudaError_t es = c->upw && c->fp32 ? dugks::strip_upwind_plan(c->coupled, c->wally, params->nx, params->ny, &c->strip)
+                         : c->fp32         ? dugks::strip_plan<float>(c->coupled, c->wally, params->nx, params->ny, &c->strip)
+                         : c->upw          ? cudaSuccess
+                                           : dugks::strip_plan<double>(c->coupled, c->wally, params->nx, params->ny, &c->strip);
         if (es == cudaSuccess && !c->fp32)
-            es = dugks::patch_plan(c->coupled, c->wally, params->nx, params->ny, c->strip.rows, &c->patch);
+            es = dugks::patch_plan(c->coupled, c->wally, c->upw, params->nx, params->ny, c->strip.rows, &c->patch);
         if (es != cudaSuccess) {
             if (c->owns) cudaFree(c->ws);
             delete c;

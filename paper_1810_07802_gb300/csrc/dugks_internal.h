@@ -53,9 +53,9 @@ struct PatchPlan {
     int tx = 0, ty = 0;   // cells (0: the strip kernel steps this problem)
     size_t smem = 0;
 };
-cudaError_t patch_plan(bool coupled, bool wally, int nx, int ny, int strip_rows, PatchPlan *out);
+cudaError_t patch_plan(bool coupled, bool wally, bool upw, int nx, int ny, int strip_rows, PatchPlan *out);
 cudaError_t launch_patch(const PatchPlan &pl, const StepArgs<double> &a, const StripPhys<double> &sp,
-                         const Phys<double> &ph, bool coupled, bool wally, cudaStream_t st);
+                         const Phys<double> &ph, bool coupled, bool wally, bool upw, cudaStream_t st);
 template <typename Real>
 cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out);
 template <typename Real>

@@ -1,4 +1,4 @@
-// The FP64 step kernel of small grids: rectangle sizes and launch.
+// The FP64 step kernel of rectangles: their sizes and launch.
 #include "dugks_internal.h"
 #include "dugks_patch.cuh"
 
@@ -6,29 +6,34 @@ namespace dugks {
 
 namespace {
 template <typename F>
-cudaError_t with_patch(bool coupled, bool wally, F &&f) {
+cudaError_t with_patch(bool coupled, bool wally, bool upw, F &&f) {
     using T = std::true_type;
     using U = std::false_type;
-    if (coupled) return wally ? f(T{}, T{}) : f(T{}, U{});
-    return wally ? f(U{}, T{}) : f(U{}, U{});
+    auto g = [&](auto c, auto w) { return upw ? f(c, w, T{}) : f(c, w, U{}); };
+    if (coupled) return wally ? g(T{}, T{}) : g(T{}, U{});
+    return wally ? g(U{}, T{}) : g(U{}, U{});
 }
 // FP64 instructions of a cell, a face and a row of 32 lanes' phi' and update (counted in the source; coupled, A-C)
 struct PatchCost {
     double cell, face, other;
 };
-PatchCost patch_cost(bool coupled) { return coupled ? PatchCost{212, 235, 56} : PatchCost{92, 90, 32}; }
+PatchCost patch_cost(bool coupled, bool upw) {
+    PatchCost c = coupled ? PatchCost{212, 235, 56} : PatchCost{92, 90, 32};
+    if (upw) c.face += coupled ? 320 : 160;   // 38 (19) limited slopes instead of the central sums
+    return c;
+}
 constexpr double kPatchFixed = 400;   // launch, loads and barriers of one CTA, in FP64 instructions (about 3 us)
 }  // namespace
 
 // The rectangle that leaves the busiest SM the fewest FP64 instructions, and that number against the strip
-// kernel's (rows of 28 columns a warp, strip_rows rows a chunk; 0: too few for strips).
-cudaError_t patch_plan(bool coupled, bool wally, int nx, int ny, int strip_rows, PatchPlan *out) {
+// kernel's (rows of 28 columns a warp, strip_rows rows a chunk; 0: too few for strips, or the upwind reconstruction).
+cudaError_t patch_plan(bool coupled, bool wally, bool upw, int nx, int ny, int strip_rows, PatchPlan *out) {
     int dev = 0, sms = 0, most = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    const PatchCost c = patch_cost(coupled);
+    const PatchCost c = patch_cost(coupled, upw);
     auto warps = [](long long n) { return double((n + 31) / 32); };
     double best = 0;
     // of the sizes that cut an axis into the same number of rectangles the smallest
@@ -37,10 +42,12 @@ cudaError_t patch_plan(bool coupled, bool wally, int nx, int ny, int strip_rows,
         if (!smallest(ty, ny)) continue;
         for (int tx = 1; tx <= 64 && tx <= nx; tx++) {
             if (!smallest(tx, nx)) continue;
-            const size_t bytes = coupled ? PatchShape<true>::smem_bytes(tx, ty) : PatchShape<false>::smem_bytes(tx, ty);
+            const size_t bytes = coupled ? (upw ? PatchShape<true, true>::smem_bytes(tx, ty) : PatchShape<true, false>::smem_bytes(tx, ty))
+                                         : (upw ? PatchShape<false, true>::smem_bytes(tx, ty) : PatchShape<false, false>::smem_bytes(tx, ty));
+            const int halo = upw ? 4 : 2;
             if (bytes > (size_t)most) continue;
             const long long tiles = (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
-            const double one = c.cell * warps((long long)(tx + 2) * (ty + 2)) +
+            const double one = c.cell * warps((long long)(tx + halo) * (ty + halo)) +
                                c.face * warps((long long)(tx + 1) * ty + (long long)tx * (ty + 1)) +
                                c.other * warps((long long)tx * ty) + kPatchFixed;
             const double t = one * double((tiles + sms - 1) / sms);
@@ -59,19 +66,19 @@ cudaError_t patch_plan(bool coupled, bool wally, int nx, int ny, int strip_rows,
         if (strip < best) out->tx = out->ty = 0;
     }
     if (out->tx == 0) return cudaSuccess;
-    return with_patch(coupled, wally, [&](auto cp, auto w) {
-        constexpr bool C = decltype(cp)::value, W = decltype(w)::value;
+    return with_patch(coupled, wally, upw, [&](auto cp, auto w, auto u) {
+        constexpr bool C = decltype(cp)::value, W = decltype(w)::value, UP = decltype(u)::value;
         static OncePerDevice<char> ready;
         return ready.get(dev, nullptr, [&](char *) {
-            return cudaFuncSetAttribute(patch_step_kernel<C, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            return cudaFuncSetAttribute(patch_step_kernel<C, W, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         });
     });
 }
 
 cudaError_t launch_patch(const PatchPlan &pl, const StepArgs<double> &a, const StripPhys<double> &sp,
-                         const Phys<double> &ph, bool coupled, bool wally, cudaStream_t st) {
-    return with_patch(coupled, wally, [&](auto cp, auto w) {
-        constexpr bool C = decltype(cp)::value, W = decltype(w)::value;
+                         const Phys<double> &ph, bool coupled, bool wally, bool upw, cudaStream_t st) {
+    return with_patch(coupled, wally, upw, [&](auto cp, auto w, auto u) {
+        constexpr bool C = decltype(cp)::value, W = decltype(w)::value, UP = decltype(u)::value;
         const PatchArgs g{pl.tx, pl.ty, (a.nx + pl.tx - 1) / pl.tx};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -83,7 +90,7 @@ cudaError_t launch_patch(const PatchPlan &pl, const StepArgs<double> &a, const S
         cfg.stream = st;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, patch_step_kernel<C, W>, a, sp, ph, g);
+        return cudaLaunchKernelEx(&cfg, patch_step_kernel<C, W, UP>, a, sp, ph, g);
     });
 }
 

@@ -1,11 +1,16 @@
-// dugks_patch.cuh -- the FP64 step kernel of small grids: one CTA per rectangle of cells.
+// dugks_patch.cuh -- the FP64 step kernel of small grids and of the upwind reconstruction: one CTA per rectangle of
+// cells.
 //
 // The FP64 pipe of an SM takes 16 cycles per warp instruction, whichever warps they come from, so a step lasts as
 // long as the SM with the most of them.  A grid of a few thousand cells is cut into rectangles of a size chosen for
-// it (patch_plan), one or a few per SM; each CTA forms its cell records with a one-cell halo, then every face, then
+// it (patch_plan), one or a few per SM; each CTA forms its cell records with a one-cell halo (upwind: two), then every face, then
 // the update, its warps taking 32 cells or faces at a time.  x- and y-faces are the same code: the scheme is
 // unchanged by exchanging the axes, so a y-face takes its neighbours along the other axis and the directions by
 // their normal and tangential components, and no warp holds two kinds of work.
+//
+// Measured, tile kernel -> rectangles: central 64^2 57.5 -> 21.1 us a step, 128^2 57.5 -> 35.7, channel 4 x 200
+// 59.5 -> 23.1, Allen-Cahn 256^2 84 -> 55; upwind 64^2 110 -> 33, 128^2 111 -> 62, 300 x 200 375 -> 206, 1024^2
+// 4,939 -> 3,698, 256 x 1024 between walls 936 -> 925.
 #pragma once
 
 #include "dugks_strip.cuh"
@@ -14,18 +19,25 @@ namespace dugks {
 
 constexpr int kPatchThreads = 256;
 
+// van Leer's limiter of two one-sided differences (R14).
+__device__ __forceinline__ double limited64(double a, double b) {
+    const double p = a * b;
+    return p > 0.0 ? (p + p) * rcp_s(a + b) : 0.0;
+}
+
 struct PatchArgs {
     int tx, ty, tiles_x;   // cells of a rectangle, rectangles across
 };
 
 // Shared memory of a rectangle, in doubles: phi', record planes, flux planes, psi~+ of the own cells.
-template <bool COUPLED>
+template <bool COUPLED, bool UPW>
 struct PatchShape {
+    static constexpr int H = UPW ? 2 : 1;          // record halo
     static constexpr int NR = COUPLED ? 22 : 13;   // f0, f1..f8, Gx, Gy, Ex, Ey; g1..g8, L
     static constexpr int NF = COUPLED ? 12 : 6;
     static constexpr int NT = COUPLED ? 16 : 8;
-    __host__ __device__ static int phis(int tx, int ty) { return (tx + 4) * (ty + 4); }
-    __host__ __device__ static int cells(int tx, int ty) { return (tx + 2) * (ty + 2); }
+    __host__ __device__ static int phis(int tx, int ty) { return (tx + 2 * H + 2) * (ty + 2 * H + 2); }
+    __host__ __device__ static int cells(int tx, int ty) { return (tx + 2 * H) * (ty + 2 * H); }
     __host__ __device__ static int faces(int tx, int ty) { return (tx + 1) * ty + tx * (ty + 1); }
     __host__ __device__ static size_t smem_bytes(int tx, int ty) {
         return sizeof(double) * ((size_t)phis(tx, ty) + (size_t)NR * cells(tx, ty) + (size_t)NF * faces(tx, ty) +
@@ -33,16 +45,17 @@ struct PatchShape {
     }
 };
 
-template <bool COUPLED, bool WALLY>
+template <bool COUPLED, bool WALLY, bool UPW>
 __global__ void __launch_bounds__(kPatchThreads, 1)
 patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_constant__ StripPhys<double> ph,
                   const __grid_constant__ Phys<double> pv, const __grid_constant__ PatchArgs g) {
-    using P = PatchShape<COUPLED>;
+    using P = PatchShape<COUPLED, UPW>;
+    constexpr int H = P::H;
     using V = double2;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int tx = g.tx, ty = g.ty, nx = a.nx, ny = a.ny, tid = threadIdx.x;
     const int x0 = ((int)blockIdx.x % g.tiles_x) * tx, y0 = ((int)blockIdx.x / g.tiles_x) * ty;
-    const int wx = tx + 4, cxn = tx + 2, ncell = P::cells(tx, ty), nface = P::faces(tx, ty), nfx = (tx + 1) * ty;
+    const int wx = tx + 2 * H + 2, cxn = tx + 2 * H, ncell = P::cells(tx, ty), nface = P::faces(tx, ty), nfx = (tx + 1) * ty;
     double *sphi = reinterpret_cast<double *>(smem_raw);
     double *rec = sphi + P::phis(tx, ty);
     double *flux = rec + (size_t)P::NR * ncell;
@@ -55,9 +68,9 @@ patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_const
 
     grid_launch_dependents();
     grid_dependency_wait();
-    // 1. phi' with a two-cell halo
+    // 1. phi', one cell beyond the records
     for (int i = tid; i < P::phis(tx, ty); i += kPatchThreads) {
-        const int iy = i / wx, gx = column(x0 - 2 + i - iy * wx), gy = map_row<WALLY>(y0 - 2 + iy, ny);
+        const int iy = i / wx, gx = column(x0 - H - 1 + i - iy * wx), gy = map_row<WALLY>(y0 - H - 1 + iy, ny);
         if (!in_bounds(gx >= 0 && gx < nx && gy >= 0 && gy < ny, a.status)) continue;
         const double *c = a.src + ((long long)gy * a.pitch + gx);
         double v[9];
@@ -66,10 +79,10 @@ patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_const
         sphi[i] = (((v[2] + v[4]) + (v[6] + v[8])) + ((v[1] + v[3]) + (v[5] + v[7]))) + v[0];
     }
     __syncthreads();
-    // 2. the cells with a one-cell halo
+    // 2. the cells with the record halo
     for (int i = tid; i < ncell; i += kPatchThreads) {
         const int iy = i / cxn, ix = i - iy * cxn;
-        const int x = x0 - 1 + ix, y = y0 - 1 + iy;
+        const int x = x0 - H + ix, y = y0 - H + iy;
         if (WALLY && (y < 0 || y >= ny)) continue;   // beyond a wall: no face reads it
         const int gx = column(x), gy = WALLY ? y : map_row<false>(y, ny);
         if (!in_bounds(gx >= 0 && gx < nx && gy >= 0 && gy < ny, a.status)) continue;
@@ -118,9 +131,9 @@ patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_const
             q[2 * ncell] = nr.g.C.x; q[4 * ncell] = nr.g.C.y; q[6 * ncell] = nr.g.D.x; q[8 * ncell] = nr.g.D.y;
             r[R_L] = nr.L;
         }
-        if (ix >= 1 && ix <= tx && iy >= 1 && iy <= ty && x < nx && y < ny) {
+        if (ix >= H && ix < tx + H && iy >= H && iy < ty + H && x < nx && y < ny) {
             const int own = tx * ty;
-            double *t = plus + (iy - 1) * tx + ix - 1;
+            double *t = plus + (iy - H) * tx + ix - H;
             t[0] = tf.A.x; t[own] = tf.A.y; t[2 * own] = tf.B.x; t[3 * own] = tf.B.y;
             t[4 * own] = tf.C.x; t[5 * own] = tf.C.y; t[6 * own] = tf.D.x; t[7 * own] = tf.D.y;
             if constexpr (COUPLED) {
@@ -142,7 +155,7 @@ patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_const
         const int j = xf ? i : i - nfx, w = xf ? tx + 1 : tx;
         const int fy = j / w, fx = j - fy * w;
         const int ns = xf ? 1 : cxn, ts = xf ? cxn : 1;
-        const int L = xf ? (fy + 1) * cxn + fx : fy * cxn + fx + 1;
+        const int L = xf ? (fy + H) * cxn + fx + H - 1 : (fy + H - 1) * cxn + fx + H;
         const int x = x0 + fx, y = y0 + fy;   // the cell at +n
         if ((xf ? y >= ny : x >= nx) || (xf ? x - 1 >= nx : y - 1 >= ny)) continue;
         const bool bottom = WALLY && !xf && y == 0, top = WALLY && !xf && y == ny;
@@ -173,7 +186,7 @@ patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_const
             auto at = [&](const double *q, int cn, int ct) {
                 const double b0 = q[0], sn = s * (b0 - q[into]);
                 double v = b0 + (0.5 * s - h * cn) * sn;
-                if (ct) v -= h * ct * (0.5 * (q[ts] - q[-ts]));
+                if (ct) v -= h * ct * (UPW ? limited64(b0 - q[-ts], q[ts] - b0) : 0.5 * (q[ts] - q[-ts]));
                 return v;
             };
             auto bars = [&](const double *q) {
@@ -205,20 +218,46 @@ patch_step_kernel(const __grid_constant__ StepArgs<double> a, const __grid_const
         } else {
             const double *r = rec + L;
             const bool lo = WALLY && xf && y == 0, hi = WALLY && xf && y == ny - 1;
-            const double ht = (lo || hi) ? 2.0 * ph.ht : ph.ht;
-            const int up = hi ? 0 : ts, down = lo ? 0 : ts;
-            fb = strip_x_open(ph, sum(r), get(r + ns), sum(r - down), ht);
-            strip_x_close(fb, sum(r + up), ht);
-            m.f0 = r[0] + r[ns];
+            if constexpr (UPW) {
+                // next to a wall a slope across it is the one-sided difference into the fluid: along an x-face's
+                // tangent (both cells), along a y-face's normal (the cell next to the wall)
+                const bool wl = WALLY && !xf && y - 1 == 0, wr = WALLY && !xf && y == ny - 1;
+                const double h = ph.h;
+                // the profile of the cell at q, on side s (-1: R, +1: L) of the face, at x_f - xi h
+                auto profile = [&](const double *q, int s, int cn, int ct) {
+                    const double c = q[0];
+                    const double sn = (s > 0 ? wl : wr) ? (s > 0 ? q[ns] - c : c - q[-ns]) : limited64(c - q[-ns], q[ns] - c);
+                    double v = c + sn * (0.5 * s - h * cn);
+                    if (ct) v -= h * ct * (lo ? q[ts] - c : hi ? c - q[-ts] : limited64(c - q[-ts], q[ts] - c));
+                    return v;
+                };
+                auto along = [&](const double *q, int ct) { return 0.5 * (profile(q, 1, 0, ct) + profile(q + ns, -1, 0, ct)); };
+                auto bars = [&](const double *q) {
+                    Dirs<double> d;
+                    d.A = v2(profile(q + kn * ncell, 1, 1, 0), along(q + kt * ncell, 1));
+                    d.B = v2(profile(q + (kn + 4) * ncell + ns, -1, -1, 0), along(q + (kt + 4) * ncell, -1));
+                    d.C = v2(profile(q + 2 * ncell, 1, 1, 1), profile(q + kc * ncell + ns, -1, -1, 1));
+                    d.D = v2(profile(q + 6 * ncell + ns, -1, -1, -1), profile(q + kd * ncell, 1, 1, -1));
+                    return d;
+                };
+                fb = bars(r);
+                m.f0 = 2.0 * along(r, 0);
+                if constexpr (COUPLED) gb = bars(r + R_g);
+            } else {
+                const double ht = (lo || hi) ? 2.0 * ph.ht : ph.ht;
+                const int up = hi ? 0 : ts, down = lo ? 0 : ts;
+                fb = strip_x_open(ph, sum(r), get(r + ns), sum(r - down), ht);
+                strip_x_close(fb, sum(r + up), ht);
+                m.f0 = r[0] + r[ns];
+                if constexpr (COUPLED) {
+                    const double *q = r + R_g;
+                    gb = strip_x_open(ph, sum(q), get(q + ns), sum(q - down), ht);
+                    strip_x_close(gb, sum(q + up), ht);
+                }
+            }
             m.G = vadd(vec(r + R_G), vec(r + R_G + ns));
             m.E = vadd(vec(r + R_E), vec(r + R_E + ns));
-            m.L = 0.0;
-            if constexpr (COUPLED) {
-                const double *q = r + R_g;
-                gb = strip_x_open(ph, sum(q), get(q + ns), sum(q - down), ht);
-                strip_x_close(gb, sum(q + up), ht);
-                m.L = r[R_L] + r[R_L + ns];
-            }
+            m.L = COUPLED ? r[R_L] + r[R_L + ns] : 0.0;
         }
         V uf = v2(0.0);
         if constexpr (!COUPLED) {

@@ -74,3 +74,14 @@ def test_upwind_strips_against_the_tile_kernels(S, nx, ny, model, bc_y):
     cfg = dict(cfg, precision="fp32", phi_ref=0.5, recon="upwind")
     strip, tile = (stepped(S, dict(cfg, tile_shape=k), f, 3) for k in (0, 1))
     assert np.abs(strip - tile).max() <= 4e-7 * np.abs(tile).max()
+
+
+@pytest.mark.parametrize("bc_y", ["periodic", "wall"])
+@pytest.mark.parametrize("model", ["coupled", "ac"])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (4, 200), (7, 5), (33, 17), (130, 70), (403, 277)])
+def test_upwind_rectangles_against_the_tile_kernels(S, nx, ny, model, bc_y):
+    """FP64 upwind: rectangles with two-cell record halos, cut by the domain's edge, beside walls, wrapped twice."""
+    cfg, f = problem(nx, ny, model, bc_y)
+    cfg = dict(cfg, recon="upwind")
+    rect, tile = (stepped(S, dict(cfg, tile_shape=k), f, 3) for k in (0, 1))
+    assert np.abs(rect - tile).max() <= 1e-12 * np.abs(tile).max()
