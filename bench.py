@@ -29,10 +29,10 @@ N_CELLS_SIDE = 2048
 FP32_BYTES_PER_CELL = 18 * 4 * 2 + 2 * 4 * 2   # read + write psi~ (18 FP32) and (phi u) history (2 FP32)
 FP64_BYTES_PER_CELL = 18 * 8 * 2 + 2 * 8 * 2
 REF_BAND_ROWS = 128
-PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "solo_step_kernel_fp32_spinodal2048.md")
-PROFILE_SUMMARY_FP64 = os.path.join(ROOT, "profiles", "solo_step_kernel_fp64_spinodal2048.md")
+PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "strip_step_kernel_fp32_spinodal2048.md")
+PROFILE_SUMMARY_FP64 = os.path.join(ROOT, "profiles", "strip_step_kernel_fp64_spinodal2048.md")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1810_07802_gb300", "csrc", f)
-                  for f in ("dugks_device.cuh", "dugks_launch.cuh")]
+                  for f in ("dugks_device.cuh", "dugks_strip.cuh", "dugks_strip_launch.cuh")]
 
 
 def parse():
@@ -577,7 +577,7 @@ def ours(args):
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak_gbs, "unit": "GB/s",
                 "frac": round(achieved / peak_gbs, 4), "traffic": traffic,
                 "algorithmic_bytes_per_launch": FP32_BYTES_PER_CELL * cells,
-                "peak_source": peak_src, "kernel": "solo_step_kernel<float,32,8,coupled,periodic>"}
+                "peak_source": peak_src, "kernel": "strip_step_kernel<float,coupled,periodic>"}
 
     extra = {}
     # second bound: instruction issue (4 schedulers per SM, one warp instruction per cycle each)
@@ -633,7 +633,7 @@ def ours(args):
         extra["upwind_fp32"] = {"value": round(cells * ku / secsu / 1e6 * world, 1), "unit": "MLUPS", "steps": ku,
                                 "ms_per_step": round(secsu / ku * 1e3, 5), "hbm_gbs": round(achu, 1),
                                 "hbm_frac": round(achu / peak_gbs, 4),
-                                "kernel": "solo_step_kernel<float,32,8,coupled,periodic,upwind>",
+                                "kernel": "strip_upwind_kernel<coupled,periodic>",
                                 "clocks": clku.summary()}
 
     line = {"metric": "coupled DUGKS MLUPS (spinodal 2048^2, FP32-shifted)", "value": round(value, 1),

@@ -9,8 +9,8 @@
 // Why a march: a tile of 32 x 8 cells computes a ring of 84 more records and 8 % of its faces twice, holds all of it
 // in shared memory between four CTA barriers, and spends a fifth of its instructions on addresses.  A strip
 // computes 32 records and 64 faces for 28 cells (14 % more than it needs; two record rows more per chunk) and
-// meets no barrier at all.  What bounds it: FP32, issue slots (any spill doubles the time, the first-level cache being
-// what the shared memory leaves); FP64, the FP64 pipe (83 % active).  Wider strips exchange columns through shared
+// meets no barrier at all.  What bounds it: FP32, issue slots (72 % active; any spill doubles the time, the first-level cache being
+// what the shared memory leaves); FP64, the FP64 pipe (85 % active).  Wider strips exchange columns through shared
 // memory behind CTA barriers: 64 to 224 columns are 5 to 80 % slower in FP32 and equal in FP64.
 //
 // Measured, tile kernel -> strip kernel: FP32 2048^2 287 -> 206 us a step, 4096^2 1,150 -> 794, 509 x 387 26.9 -> 16.6,
