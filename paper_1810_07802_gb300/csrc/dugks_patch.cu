@@ -26,7 +26,7 @@ constexpr double kPatchFixed = 400;   // launch, loads and barriers of one CTA, 
 }  // namespace
 
 // The rectangle that leaves the busiest SM the fewest FP64 instructions, and that number against the strip
-// kernel's (rows of 28 columns a warp, strip_rows rows a chunk; 0: too few for strips, or the upwind reconstruction).
+// kernel's (rows of 28 columns a warp, strip_rows rows a chunk; 0: no strips for this problem).
 cudaError_t patch_plan(bool coupled, bool wally, bool upw, int nx, int ny, int strip_rows, PatchPlan *out) {
     int dev = 0, sms = 0, most = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -1,5 +1,5 @@
-// dugks_patch.cuh -- the FP64 step kernel of small grids and of the upwind reconstruction: one CTA per rectangle of
-// cells.
+// dugks_patch.cuh -- the FP64 step kernel of small grids, of the coupled model between walls and of the upwind
+// reconstruction: one CTA per rectangle of cells.
 //
 // The FP64 pipe of an SM takes 16 cycles per warp instruction, whichever warps they come from, so a step lasts as
 // long as the SM with the most of them.  A grid of a few thousand cells is cut into rectangles of a size chosen for
@@ -10,7 +10,8 @@
 //
 // Measured, tile kernel -> rectangles: central 64^2 57.5 -> 21.1 us a step, 128^2 57.5 -> 35.7, channel 4 x 200
 // 59.5 -> 23.1, Allen-Cahn 256^2 84 -> 55; upwind 64^2 110 -> 33, 128^2 111 -> 62, 300 x 200 375 -> 206, 1024^2
-// 4,939 -> 3,698, 256 x 1024 between walls 936 -> 925.
+// 4,939 -> 3,698, 256 x 1024 between walls 936 -> 925; coupled central between walls, strips -> rectangles: 380^2 382 ->
+// 255 (tiles 371), 1024^2 2,211 -> 1,844, 3000 x 200 1,453 -> 1,023.
 #pragma once
 
 #include "dugks_strip.cuh"

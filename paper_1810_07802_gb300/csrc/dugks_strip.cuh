@@ -86,7 +86,7 @@ struct StripShape {
     static constexpr int S = sizeof(Real) == 4 && !KEEP ? 4 : 3;   // staged rows in flight or in use
     static constexpr int KG = COUPLED ? 13 : 8;    // kept groups of 4 values: psi~+ of two rows, one flux
     static constexpr int AL = 128 / int(sizeof(Real));
-    static constexpr int RG = SHF ? 0 : (COUPLED ? 6 : 4);   // record groups of 4 values (exchanged by shuffles: none)
+    static constexpr int RG = SHF ? 0 : 4;   // record groups of 4 values (exchanged by shuffles: none)
     __host__ __device__ static constexpr int up(int v) { return (v + AL - 1) / AL * AL; }
     // columns of a staged row: x0 - 4 .. x0 - 4 + box - 1
     __host__ __device__ static constexpr int box(int w) { return w + 4; }
@@ -103,7 +103,7 @@ struct StripShape {
         return off_rec(w) + rec_rows(wally) * rec_stride(w);
     }
     __host__ __device__ static constexpr int off_phi(int w, bool wally) {
-        return off_flux(w, wally) + (SHF ? 0 : up((COUPLED ? 12 : 6) * (w + 1) + 4));
+        return off_flux(w, wally) + (SHF ? 0 : up(6 * (w + 1) + 4));
     }
     __host__ __device__ static constexpr int off_bar(int w, bool wally) { return off_phi(w, wally) + (SHF ? 0 : up(w + 2)) + (KEEP ? KG * 4 * w : 0); }
     __host__ __device__ static constexpr size_t smem_bytes(int w, bool wally) {
@@ -111,8 +111,8 @@ struct StripShape {
     }
 };
 
-// Columns are exchanged by shuffles; in FP64 with walls through shared memory (the wall faces read the records of
-// two rows from there).
+// Columns are exchanged by shuffles; in FP64 with walls (Allen-Cahn alone) through shared memory (the wall faces read
+// the records of two rows from there).
 template <typename Real, bool WALLY>
 __host__ __device__ constexpr bool strip_shuffles() {
     return !WALLY || sizeof(Real) == 4;
@@ -697,6 +697,7 @@ template <typename Real, bool COUPLED, bool WALLY>
 __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<Real> &a, const StripPhys<Real> &ph,
                                             const Phys<Real> &pv, int x0, int ya, int yb) {
     constexpr bool SHF = strip_shuffles<Real, WALLY>();
+    static_assert(SHF || !COUPLED, "shared memory holds the records of f alone");
     using S = StripShape<Real, COUPLED, SHF, false>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Real *sm = reinterpret_cast<Real *>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
@@ -800,7 +801,6 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
     advance();
     __syncwarp();
     const int gCDf = 0, gABf = 4 * (W + 2), gAux = 8 * (W + 2), gRest = 12 * (W + 2);
-    const int gCDg = 16 * (W + 2), gABg = 20 * (W + 2);
     const int last = yb - ya + 1;
     for (int j = 0; j <= last; j++) {
         const int r = ya - 1 + j;
@@ -851,10 +851,6 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
                 st_pairs(rec + 4 + gAux, nr.G, nr.E);
                 st2(rec + 4 + gRest, nr.f0, nr.L);
             }
-            if constexpr (COUPLED && !SHF) {
-                st_pairs(rec + 4 + gCDg, nr.g.C, nr.g.D);
-                st_pairs(rec + 4 + gABg, nr.g.A, nr.g.B);
-            }
         }
         __syncwarp();
         load_row(j + 1 + S::S, cslot);   // the slot of row r is free: every thread has read it
@@ -903,20 +899,6 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
                 Rf.D = vsub(e.D, q.D);
                 Rf.A.x = e.A.x - q.A.x;
                 Rf.B.x = e.B.x - q.B.x;
-                if constexpr (COUPLED) {
-                    ld_pairs(rec + gCDg, q.C, q.D);
-                    ld_pairs(rec + gABg, q.A, q.B);
-                    nSg.A = vadd(q.A, nr.g.A);
-                    nSg.B = vadd(q.B, nr.g.B);
-                    nSg.C = vadd(q.C, nr.g.C);
-                    nSg.D = vadd(q.D, nr.g.D);
-                    ld_pairs(rec + 8 + gCDg, e.C, e.D);
-                    ld_pairs(rec + 8 + gABg, e.A, e.B);
-                    Rg.C = vsub(e.C, q.C);
-                    Rg.D = vsub(e.D, q.D);
-                    Rg.A.x = e.A.x - q.A.x;
-                    Rg.B.x = e.B.x - q.B.x;
-                }
             }
         }
         const Real half = Real(0.5);
@@ -946,12 +928,7 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
             xf = strip_face<Real, COUPLED, true>(ph, Xf, Xg, Xm, false, uf);
             if constexpr (!SHF) {
                 st_pairs(sflx, xf.fC, xf.fD);
-                if constexpr (COUPLED) {
-                    st_pairs(sflx + 4 * (W + 1), xf.gC, xf.gD);
-                    st_pairs(sflx + 8 * (W + 1), xf.fn, xf.gn);
-                } else {
-                    st2(sflx + 4 * (W + 1) - 2 * tid, xf.fn.x, xf.fn.y);
-                }
+                st2(sflx + 4 * (W + 1) - 2 * tid, xf.fn.x, xf.fn.y);
             }
         }
         // the x-face of row r, opened (next to a wall the slope is one-sided: the row takes itself as the one
@@ -998,11 +975,8 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
                     const int j0 = j - 1, j1 = TOP ? j - 2 : j;   // iterations whose records to take
                     const Real *row = srec + (j0 & 1) * S::rec_stride(W) + 4 * (tid + 1);
                     const Real *into = srec + (j1 & 1) * S::rec_stride(W) + 4 * (tid + 1);
-                    Real rest, unused = Real(0);
-                    const Dirs<Real> fb = strip_wall<Real, TOP>(row, into, gCDf, gABf, ph, row[gRest], into[gRest], rest);
-                    Dirs<Real> gb;
-                    if constexpr (COUPLED)
-                        gb = strip_wall<Real, TOP>(row, into, gCDg, gABg, ph, Real(0), Real(0), unused);
+                    Real rest;
+                    const Dirs<Real> fb = strip_wall<Real, TOP>(row, into, gCDf, gABf, ph, row[gRest], into[gRest], rest), gb{};
                     FaceSum<Real> m;   // the cell and its mirror image
                     m.f0 = Real(2) * rest;
                     m.L = Real(2) * row[gRest + 1];
@@ -1041,12 +1015,6 @@ __device__ __forceinline__ void strip_march(const StripMaps &tm, const StepArgs<
                 }
             } else {
                 ld_pairs(p, xe.fC, xe.fD);
-            }
-            if constexpr (SHF) {
-            } else if constexpr (COUPLED) {
-                ld_pairs(p + 4 * (W + 1), xe.gC, xe.gD);
-                ld_pairs(p + 8 * (W + 1), xe.fn, xe.gn);
-            } else {
                 Real z[2];
                 ld2(sflx + 4 * (W + 1) - 2 * tid + 2, z);
                 xe.fn = v2(z[0], z[1]);

@@ -8,12 +8,20 @@
 
 namespace dugks {
 
-template <typename F>
+// FP64 has no strips for the coupled model between walls: the records that its wall faces read from shared memory leave
+// room for one warp a scheduler, and the rectangles are faster at every size (380^2 255 us a step against the strips'
+// 382 and the tiles' 371, 5000 x 40 348, 552 and 513, 1400^2 3,376, 3,993 and 4,620).
+template <typename Real>
+constexpr bool strip_compiled(bool coupled, bool wally) { return sizeof(Real) == 4 || !coupled || !wally; }
+
+template <typename Real, typename F>
 cudaError_t with_strip(bool coupled, bool wally, F &&f) {
     using T = std::true_type;
     using U = std::false_type;
-    if (coupled) return wally ? f(T{}, T{}) : f(T{}, U{});
-    return wally ? f(U{}, T{}) : f(U{}, U{});
+    if (!coupled) return wally ? f(U{}, T{}) : f(U{}, U{});
+    if constexpr (strip_compiled<Real>(true, true))
+        if (wally) return f(T{}, T{});
+    return wally ? cudaErrorInvalidValue : f(T{}, U{});
 }
 
 // Shared memory of a CTA of which 4 w and no more fit on an SM (228 KB, 1 KB of each CTA the system's).
@@ -54,8 +62,8 @@ cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out)
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    return with_strip(coupled, wally, [&](auto c, auto wl) {
+    if (e != cudaSuccess || !strip_compiled<Real>(coupled, wally)) return e;
+    return with_strip<Real>(coupled, wally, [&](auto c, auto wl) {
         constexpr bool C = decltype(c)::value, W = decltype(wl)::value;
         using S = StripShape<Real, C, strip_shuffles<Real, W>(), strip_keeps<Real, W>()>;
         constexpr size_t bytes = S::smem_bytes(kStripLanes, W);
@@ -84,7 +92,8 @@ cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out)
         // 162 against 137).  Below one warp a scheduler there is nothing to even out (64^2 5.0 against 6.0).
         const bool even = per_sm > 4 * w && (long long)nstrips * ((ny + rows - 1) / rows) > 4ll * sms;
         out->smem = even ? std::max(bytes, strip_share(w)) : bytes;
-        // FP64: below eight rows a chunk the tile kernel's halo costs less than the rows a chunk adds
+        // FP64: below eight rows a chunk the rectangles are faster at every size measured, 1.2 to 1.9 times where the grid
+        // fills the chip (380^2 257 us a step against 329, Allen-Cahn 116 against 145) and up to 4.1 on smaller ones
         if (sizeof(Real) == 8 && rows < 8) return cudaSuccess;
         out->threads = kStripLanes;
         out->box = S::box(kStripLanes);
@@ -98,7 +107,7 @@ cudaError_t strip_plan(bool coupled, bool wally, int nx, int ny, StripPlan *out)
 template <typename Real>
 cudaError_t launch_strip(const StripPlan &pl, const StripMaps &tm, const StepArgs<Real> &a, const typename StripConst<Real>::T &sp,
                          const Phys<Real> &ph, bool coupled, bool wally, cudaStream_t st) {
-    return with_strip(coupled, wally, [&](auto c, auto wl) {
+    return with_strip<Real>(coupled, wally, [&](auto c, auto wl) {
         constexpr bool C = decltype(c)::value, W = decltype(wl)::value;
         using S = StripShape<Real, C, strip_shuffles<Real, W>(), strip_keeps<Real, W>()>;
         const StripArgs g{pl.nstrips, pl.rows};
@@ -149,7 +158,7 @@ cudaError_t launch_strip_group(const StripInst<Real> *inst, const typename Strip
         g.first[i + 1] = g.first[i] + members[i].x * ((members[i].y + rows - 1) / rows);
         g.ph[i] = ph[i];
     }
-    return with_strip(coupled, wally, [&](auto c, auto wl) {
+    return with_strip<Real>(coupled, wally, [&](auto c, auto wl) {
         constexpr bool C = decltype(c)::value, W = decltype(wl)::value;
         using S = StripShape<Real, C, strip_shuffles<Real, W>(), strip_keeps<Real, W>()>;
         cudaLaunchAttribute at[1];
