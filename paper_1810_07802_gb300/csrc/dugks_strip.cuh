@@ -202,13 +202,23 @@ inline StripPhys<Real> strip_phys(const Phys<double> &p) {
 
 // FP64: the hardware's 20-bit seed refined once at third order: with e = 1 - x y the series 1 / x = y (1 + e + e^2 +
 // ...), with e = 1 - x y^2 the series 1 / sqrt(x) = y (1 + e / 2 + 3 e^2 / 8 + ...); what is left is of order e^3.
+// Within 1 ulp for arguments of 2^-1021 to 2^1021.  Where the seed is 0, infinite or NaN (x infinite, zero, outside
+// that range or NaN) it is the result, as of a division; the test is integer work, which the FP64 pipe does not see.
+__device__ __forceinline__ bool seed_is_result(double y) {
+#ifdef __CUDA_ARCH__
+    const unsigned m = (unsigned)__double2hiint(y) & 0x7fffffffu;
+    return m - 0x00100000u >= 0x7fe00000u;
+#else
+    return false;
+#endif
+}
 __device__ __forceinline__ double rcp_s(double x) {
     double y = x;
 #ifdef __CUDA_ARCH__
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
 #endif
     const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    return seed_is_result(y) ? y : fma(y, fma(e, e, e), y);
 }
 __device__ __forceinline__ double rsqrt_s(double x) {
     double y = x;
@@ -216,7 +226,7 @@ __device__ __forceinline__ double rsqrt_s(double x) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
 #endif
     const double e = fma(-(x * y), y, 1.0);
-    return fma(y, e * fma(0.375, e, 0.5), y);
+    return seed_is_result(y) ? y : fma(y, e * fma(0.375, e, 0.5), y);
 }
 
 // State at a cell or a face (units of G, L and E above).
