@@ -167,9 +167,10 @@ struct Pt {
     Real Dx, Dy;
 };
 
-// FP32 takes the hardware's approximations as they are: their arguments (|grad phi|^2 + 1e-16, densities,
-// viscosities, relaxation times) stay clear of the denormals and of 2^126, where alone rsqrtf and __fdividef
-// (1, x) rescale around the same instructions.  FP64: rsqrt and IEEE division.
+// FP32 takes the hardware's approximations: reciprocal within 1 ulp, inverse root within 2^-22.9, for normal
+// arguments below 2^126 (denormals count as zero).  The arguments here (|grad phi|^2 + 1e-16, densities, viscosities,
+// relaxation times) are of that range, over which both were found equal to rsqrtf(x) and __fdividef(1, x).  FP64:
+// rsqrt and IEEE division.
 __device__ __forceinline__ float rsqrt_r(float x) {
     float y = x;
 #ifdef __CUDA_ARCH__

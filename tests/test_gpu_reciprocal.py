@@ -2,7 +2,8 @@
 ends, and what a caller sees of them where a density is zero.
 
 Bounds.  rcp_s: the refined value is rounded once, what the series leaves is of order 2^-60: 1 ulp.  rsqrt_s: half an
-ulp from the last rounding, half at most from that of x y: 1 ulp and the same remainder, 1.1."""
+ulp from the last rounding, half at most from that of x y: 1 ulp and the same remainder, 1.1.  FP32: those that the
+PTX documentation states for the instructions, 1 ulp and 2^-22.9."""
 import ctypes
 import os
 import subprocess
@@ -22,12 +23,20 @@ template <typename F, typename T> __global__ void map(F f, const T *x, T *y, int
 }
 struct Rcp64 { __device__ double operator()(double v) const { return dugks::rcp_s(v); } };
 struct Root64 { __device__ double operator()(double v) const { return dugks::rsqrt_s(v); } };
+struct Rcp32 { __device__ float operator()(float v) const { return dugks::rcp_r(v); } };
+struct Root32 { __device__ float operator()(float v) const { return dugks::rsqrt_r(v); } };
+struct CudaRcp32 { __device__ float operator()(float v) const { return __fdividef(1.0f, v); } };
+struct CudaRoot32 { __device__ float operator()(float v) const { return rsqrtf(v); } };
 template <typename F, typename T> int run(F f, const T *x, T *y, int n) {
     map<<<(n + 255) / 256, 256>>>(f, x, y, n);
     return (int)cudaDeviceSynchronize();
 }
 extern "C" int rcp64(const double *x, double *y, int n) { return run(Rcp64(), x, y, n); }
 extern "C" int root64(const double *x, double *y, int n) { return run(Root64(), x, y, n); }
+extern "C" int rcp32(const float *x, float *y, int n) { return run(Rcp32(), x, y, n); }
+extern "C" int root32(const float *x, float *y, int n) { return run(Root32(), x, y, n); }
+extern "C" int cuda_rcp32(const float *x, float *y, int n) { return run(CudaRcp32(), x, y, n); }
+extern "C" int cuda_root32(const float *x, float *y, int n) { return run(CudaRoot32(), x, y, n); }
 """
 
 
@@ -84,6 +93,17 @@ def test_fp64_at_the_ends_of_the_range(call):
     assert np.array_equal(got, want, equal_nan=True) and np.array_equal(np.signbit(got[:4]), np.signbit(want[:4]))
     x = np.array([0.0, np.inf, np.nan, -1.0])
     assert np.array_equal(call("root64", x), np.array([np.inf, 0.0, np.nan, np.nan]), equal_nan=True)
+
+
+def test_fp32(call):
+    x = arguments(-126, 126, np.float32)
+    got = call("rcp32", x)
+    assert ulps(got, 1 / x.astype(np.float64), np.float32) <= 1.0
+    assert np.array_equal(got, call("cuda_rcp32", x))
+    got = call("root32", x)
+    exact = 1 / np.sqrt(x.astype(np.float64))
+    assert float(np.max(np.abs(got - exact) / exact)) <= 2.0 ** -22.9
+    assert np.array_equal(got, call("cuda_root32", x))
 
 
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
