@@ -664,6 +664,12 @@ dugks_status dugks_set_rows(dugks_handle c, int32_t row0, int32_t nrows, const v
 
 int64_t dugks_step_count(dugks_handle c) { return c ? c->steps : -1; }
 
+int32_t dugks_step_kernel(dugks_handle c, int32_t *strip_rows) {
+    if (!c) return -1;
+    if (strip_rows) *strip_rows = c->strip.threads ? c->strip.rows : 0;
+    return c->patch.tx ? 2 : c->strip.threads ? 1 : 0;
+}
+
 dugks_status dugks_sync(dugks_handle c) {
     if (!c) return DUGKS_ERR_ARG;
     return sync_status(c);

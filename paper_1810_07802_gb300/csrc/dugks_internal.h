@@ -178,6 +178,11 @@ struct dugks_ctx {
     }
 };
 
+// Which kernel dugks_step runs for a problem: 0 tiles, 1 strips, 2 rectangles (-1: no handle).  *strip_rows: rows of
+// a strip's chunk, 0 where the problem has no strips (a batch takes strips where it has).  For the tests: not part of
+// the C ABI.
+extern "C" int32_t dugks_step_kernel(dugks_handle c, int32_t *strip_rows);
+
 namespace dugks {
 // Enqueues nsteps single-problem steps of c on stream st and advances its
 // step count and ping-pong index (dugks_step on the handle's own stream; a
