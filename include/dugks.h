@@ -250,8 +250,9 @@ dugks_status dugks_get_distributions(dugks_handle h, double *f, double *g, doubl
  * solver's stream, no synchronisation) or host memory (synchronises).  Rows
  * written this way replace the state the next step reads; a band stepped
  * with its halo rows refreshed from its neighbours before every step gives
- * its own rows the bits of the single-domain step.  DUGKS_ERR_ARG for rows
- * outside the grid. */
+ * its own rows the values of the single-domain step to round-off (a band may
+ * be stepped by another kernel than the whole domain, see tile_shape, or be
+ * cut otherwise by the same one).  DUGKS_ERR_ARG for rows outside the grid. */
 size_t dugks_state_element_bytes(dugks_handle h);
 dugks_status dugks_get_rows(dugks_handle h, int32_t row0, int32_t nrows, void *buf, int32_t buf_is_device);
 dugks_status dugks_set_rows(dugks_handle h, int32_t row0, int32_t nrows, const void *buf, int32_t buf_is_device);

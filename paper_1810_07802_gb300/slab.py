@@ -9,7 +9,9 @@ further out (the gradient and Laplacian of Sec. II.B) and g and
 reads the profile of the cell a direction leaves, one row further again:
 three halo rows.  Before every step a band takes from each neighbour that
 neighbour's `halo` edge rows of every stored plane, and its own rows then get
-the bits of the single-domain step.
+the values of the single-domain step: to round-off from the GPU solver, which
+chooses its step kernel by the size of the grid it is given, and bit for bit
+from a stepper that computes every cell alike.
 
 Boundaries.  A y-periodic problem is cut into bands that are periodic
 problems of their own rows plus a halo on both sides; the wrap-around of a
