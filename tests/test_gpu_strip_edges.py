@@ -106,3 +106,13 @@ def test_more_members_than_one_launch_carries(S, model, bc_y):
         for (cfg, f), got in zip(problems, stepped_together(S, problems, 3, True)):
             ref = tiles(S, cfg, f, 3)
             assert np.abs(got - ref).max() <= 4e-7 * np.abs(ref).max(), (cfg["nx"], cfg["ny"])
+
+
+@pytest.mark.parametrize("precision,model,bc_y", [("fp64",) + k for k in KINDS] + [("fp32", "coupled", "periodic"),
+                                                                                   ("fp32", "coupled", "wall")])
+def test_chunk_heights_of_a_group_change_no_bits(S, precision, model, bc_y):
+    """The rows of a chunk are chosen for a whole group: a member alone has others, and the same bits."""
+    problems = [problem(nx, ny, model, bc_y, precision) for nx, ny in ((496, 512), (32, 8171), (31, 7999))]
+    together = stepped_together(S, problems, 5, True)
+    for p, got in zip(problems, together):
+        assert np.array_equal(got, stepped_together(S, [p], 5, True)[0]), (p[0]["nx"], p[0]["ny"])
