@@ -171,12 +171,14 @@ dugks_status dugks_check_batch_wait(int64_t budget_ns, void *cuda_stream);
  * unknown precision.  Shape 1 is the tile kernels' default.  No device work. */
 int32_t dugks_tile_shapes(int32_t precision, int32_t *tx, int32_t *ty, int32_t cap);
 
-/* Autotuner of the step kernel's tile shape for one problem.  For every
+/* Autotuner of the tile kernels' shape for one problem.  It does not time
+ * tile_shape 0, the library's choice, whose kernels step most problems faster
+ * than any tile: to pin its result, compare it with 0 first.  For every
  * compiled shape it creates the problem (params, with tile_shape replaced,
  * and the host fields as for dugks_create) in a library-allocated workspace,
  * runs 2 warm-up steps, times trial_steps (>= 1) steps with CUDA events on
  * cuda_stream and destroys it; one shape at a time, so the device memory
- * needed is one workspace.  Writes the fastest tile_shape value (>= 1) to
+ * needed is one workspace.  Writes the fastest of them (>= 1) to
  * *best and, if ms_per_step is not NULL, the milliseconds per step of shape
  * k to ms_per_step[k - 1] (-1 where a shape failed; as many entries as
  * dugks_tile_shapes returns).  Synchronises.  Returns DUGKS_OK if at least

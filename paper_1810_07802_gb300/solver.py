@@ -171,8 +171,8 @@ def check_batch_wait(budget_ns=0, stream=None):
 
 
 def tile_shapes(precision="fp32"):
-    """Compiled step-kernel tile shapes [(tx, ty), ...]; cfg["tile_shape"] = k
-    selects entry k - 1 (0: the library default, entry 0)."""
+    """Compiled shapes of the tile kernels [(tx, ty), ...]; cfg["tile_shape"] =
+    k selects entry k - 1 (0: the library's choice among all step kernels)."""
     prec = _ENUM["precision"][precision]
     n = int(lib().dugks_tile_shapes(prec, None, None, 0))
     tx, ty = (ctypes.c_int32 * n)(), (ctypes.c_int32 * n)()
@@ -183,7 +183,9 @@ def tile_shapes(precision="fp32"):
 def autotune(cfg, phi0, ux0=None, uy0=None, p0=None, trial_steps=20, stream=None):
     """Times every compiled tile shape on this problem (one at a time, in
     library-allocated workspaces) and returns (best tile_shape value,
-    [ms per step of each shape, -1 where one failed])."""
+    [ms per step of each shape, -1 where one failed]).  tile_shape 0, the
+    library's choice, is not timed and mostly faster (serve.tuned_shape
+    compares it too)."""
     import torch
 
     params = make_params(cfg)
