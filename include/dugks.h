@@ -92,11 +92,12 @@ typedef struct {
     int32_t visc_interp;   /* dugks_visc: 1/mu linear in phi (Eq. 35) or mu (Eq. 36) */
     int32_t gravity_mode;  /* 0: G = (gx, gy); 1: G = (rho - rho_ref)(gx, gy)      */
     int32_t tile_shape;    /* 0: the library's choice of step kernel (one warp
-                              marching up a strip of columns, rectangles for
-                              small or upwind FP64 grids); k >= 1: the tile
-                              kernel of the k-th compiled shape of the precision
-                              (see dugks_tile_shapes, dugks_autotune).  All
-                              compute the same scheme                              */
+                              marching up a strip of columns; rectangles for
+                              FP64 grids that are small, upwind or coupled
+                              between walls); k >= 1: the tile kernel of the
+                              k-th compiled shape of the precision (see
+                              dugks_tile_shapes, dugks_autotune).  All compute
+                              the same scheme                                      */
     double cfl;            /* dt = cfl (Eq. 37 with delta_x = 1, RT = 1/3), > 0    */
     double mobility;       /* M_phi > 0; tau_f = M_phi / RT (Eq. 34)               */
     double width;          /* interface width W > 0 (Eq. 3)                        */
@@ -290,13 +291,15 @@ dugks_status dugks_destroy(dugks_handle h);
  * members of uneven size advance without a batch-wide barrier between steps.
  * Either way the launches are captured once into CUDA graphs (16 steps, and
  * one step) and replayed until the membership changes.  The two modes run
- * separately compiled kernels and agree to round-off.  Each CTA runs the same tile code as
- * dugks_step, with the member's constants read from a device descriptor
- * instead of the kernel's parameter space, so the two agree to round-off.  A
- * member of 2048 tiles or more fills the GPU by itself: it is stepped by
- * dugks_step's kernel on the batch's stream and is bit-identical to stepping
- * it alone.  Which path a member takes depends on its own size only, so its
- * result does not depend on the rest of the batch.
+ * separately compiled kernels and agree to round-off.  A group's kernel is a
+ * strip kernel where the member has strips (FP32 central, large FP64 central
+ * grids) and a tile kernel elsewhere (explicit tile shapes, upwind, small or
+ * walled coupled FP64 grids), also where dugks_step takes another kernel for
+ * the same problem: the two agree to round-off.  A member of 2048 tiles or
+ * more fills the GPU by itself: it is stepped by dugks_step's kernel on the
+ * batch's stream and is bit-identical to stepping it alone.  Which path a
+ * member takes depends on its own parameters and size only, so its result does
+ * not depend on the rest of the batch.
  * Members may differ in size, physics and precision.  While a handle is in a
  * batch, advance it only through the batch; its other calls (dugks_macros,
  * dugks_reduce, ...) stay valid but run on the handle's own stream, so use

@@ -1,14 +1,16 @@
 // dugks_batch.cu -- batches of independent solvers advanced together.
 //
 // Members are grouped by kernel variant (precision x model x y-boundary x
-// tile shape x reconstruction).
-// Each group owns a device array of per-problem descriptors (buffers,
-// constants, tensor maps, step counter), a work list of (problem, tile)
-// items and 1 + members counters.  By default K steps of a group are one
-// persistent launch (a queue of K x items taken in step order; a tile waits
-// only for its own member's previous step, counted per member) plus a tiny
-// launch that advances every member's buffer parity and step count; the
-// other mode launches one grid per step.  The launches of K steps are
+// tile shape x reconstruction).  Members that have strips form strip groups:
+// one launch a step over all (problem, strip chunk) items of up to 64 members,
+// each launch overlapping the end of the one before.  The others form tile
+// groups: a device array of per-problem descriptors (buffers, constants,
+// tensor maps, step counter), a work list of (problem, tile) items and 1 +
+// members counters; one grid launch a step, or, in the persistent mode, K
+// steps in one launch (a queue of K x items taken in step order; a tile waits
+// only for its own member's previous step, counted per member).  Either ends
+// with a tiny launch that advances every member's buffer parity and step
+// count.  The launches of K steps, every group a branch of its own, are
 // captured once into a CUDA graph and replayed until membership changes (one
 // graph of 16 steps and one of a single step).
 //

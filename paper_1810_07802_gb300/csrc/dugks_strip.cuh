@@ -4,14 +4,14 @@
 // psi~+ partials of Eq. 30), the west x-face and the y-face to the row below, and finishes the row below with the
 // flux update (Eq. 24).  What a row needs from the rows around it stays in the lane's registers; what it needs from
 // the columns beside it comes by shuffles.  A grid is cut into strips of 28 columns and chunks of rows, as many as
-// run at once (strip_plan); rows arrive by TMA three ahead of use and leave by TMA stores.
+// run at once (strip_plan); rows arrive by TMA two ahead of use (FP32 between walls three) and leave by TMA stores.
 //
 // Why a march: a tile of 32 x 8 cells computes a ring of 84 more records and 8 % of its faces twice, holds all of it
 // in shared memory between four CTA barriers, and spends a fifth of its instructions on addresses.  A strip
 // computes 32 records and 64 faces for 28 cells (14 % more than it needs; two record rows more per chunk) and
-// meets no barrier at all.  What bounds it: FP32, issue slots (72 % active; any spill doubles the time, the first-level cache being
-// what the shared memory leaves); FP64, the FP64 pipe (85 % active).  Wider strips exchange columns through shared
-// memory behind CTA barriers: 64 to 224 columns are 5 to 80 % slower in FP32 and equal in FP64.
+// meets no barrier at all.  What bounds it: FP32, issue slots (72 % active; any spill doubles the time, the first-level
+// cache being what the shared memory leaves); FP64, the FP64 pipe (85 % active).  Wider strips exchange columns through
+// shared memory behind CTA barriers: 64 to 224 columns are 5 to 80 % slower in FP32 and equal in FP64.
 //
 // Measured, tile kernel -> strip kernel: FP32 2048^2 287 -> 206 us a step, 4096^2 1,150 -> 794, 509 x 387 26.9 -> 16.6,
 // 64^2 10.3 -> 5.0, 256 x 1024 between walls 28.9 -> 21.4; FP64 1024^2 2,464 -> 1,757.

@@ -131,10 +131,11 @@ class BatchingServer:
     hbm_budget: bytes of solver workspaces that may be resident at once.
     max_members: slots (resident problems) at most.
     chunk: steps enqueued between scheduling decisions at most.
-    tile_policy: None (the library's default tile shape) or a callable
+    tile_policy: None (the library's choice of step kernel) or a callable
       (cfg, fields) -> tile_shape, e.g. an AutotuneCache.
-    persistent: advance the batch in persistent launches of up to 16 steps
-      (dugks_batch_set_persistent) instead of one grid launch per step.
+    persistent: advance the members that tile kernels step in persistent
+      launches of up to 16 steps (dugks_batch_set_persistent) instead of one
+      grid launch per step.
     """
 
     def __init__(self, hbm_budget, max_members=128, chunk=50, stream=None, solver_factory=None,

@@ -413,8 +413,9 @@ class Solver:
 
 class Batch:
     """Members (Solver objects) advanced together by dugks_batch_step.
-    persistent: K steps of each kernel group per launch, else (the default)
-    one grid launch per group and step (dugks_batch_set_persistent)."""
+    persistent: K steps of each group of tile kernels per launch, else (the
+    default, and always for strips) one grid launch per group and step
+    (dugks_batch_set_persistent)."""
 
     def __init__(self, stream=None, persistent=False):
         import torch
